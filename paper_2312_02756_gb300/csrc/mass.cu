@@ -18,7 +18,7 @@
 #include "common.cuh"
 #include "mass_lc.cuh"
 #include "mass_lc_grad.cuh"
-#include "pair_math.cuh"
+#include "pair_raw.cuh"
 
 namespace gvx {
 namespace {
@@ -53,16 +53,6 @@ __global__ void __launch_bounds__(256) mass_kernel(Lv a, Lv b, T *__restrict__ m
   }
 }
 
-// One FP64 pair: the light-cone float-float fast path (mass_lc.cuh), the FP64 formulas for a
-// lane outside its domain.
-__device__ __forceinline__ double pair_mass_f64(const V4<double> &x, const V4<double> &y,
-                                                const ffm::LcTab &T) {
-  double out;
-  if (!ffm::pair_mass_lc(x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, T, &out))
-    out = sqrt(pair_terms(make_leg(x), make_leg(y)).m2);
-  return out;
-}
-
 // FP64 forward: grid-stride, one pair per thread and step; 64 registers, eight CTAs of 128
 // threads per SM, a grid of 32 times the resident CTAs (small CTAs and many waves even out the
 // SMs' progress: 2-3% faster than four CTAs of 256 and 8 waves on GB300).  For a leg in SoA layout (four separate arrays), lanes 0..7 of each warp
@@ -83,7 +73,7 @@ __global__ void __launch_bounds__(128, 8) mass_f64_kernel(Lv a, Lv b, double *__
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const int64_t next = i - lane + stride;  // the warp's first element of the next step
     if (prefetch && next + 32 <= n) asm volatile("prefetch.global.L2 [%0];" ::"l"(pbase + 8 * next));
-    st_s(m + i, pair_mass_f64(ld4<double, LA>(a, i), ld4<double, LB>(b, i), T));
+    st_s(m + i, pair_mass_raw(ld4<double, LA>(a, i), ld4<double, LB>(b, i), T));
   }
 }
 

@@ -142,9 +142,7 @@ GVX_HD ff cvt1(const CvtParts &a) { return {u2f(a.hb), fsub(u2f(a.ab), u2f(a.bb)
 // ---- lane-generic float-float steps ---------------------------------------------------------
 // Each step is written once for V = float (one value) and V = f2 (two values as the lanes of
 // Blackwell's paired FP32 instructions).  A lane of the paired form rounds exactly as the scalar
-// form (a - b and -a are single correctly rounded or exact operations either way), so the
-// jagged kernel's per-particle terms (scalar) have the bits of the elementwise kernel's two
-// legs (paired).  Results may be unnormalized: |lo| up to ~2 ulp(hi).
+// form (a - b and -a are single correctly rounded or exact operations either way).  Results may be unnormalized: |lo| up to ~2 ulp(hi).
 
 GVX_HD float fmin_(float a, float b) { return a < b ? a : b; }
 GVX_HD float vadd(float a, float b) { return fadd(a, b); }
@@ -352,13 +350,12 @@ template <class F>
 struct LcLeg {
   F P, E, Y, D;
 };
-// With sh (chp) given, also *sh = sinh(x) (*chp = cosh(x)), from the same reduction and entry.
+// The terms from |eta| already reduced to n 2^-8 + r.  With sh (chp) given, also *sh = sinh(x)
+// (*chp = cosh(x)), from the same entry.
 template <class F>
-GVX_HD LcLeg<F> lc_leg(const F &pt, const F &mm, const F &x, const gvx_f4 *hyp, F *sh = nullptr,
-                       F *chp = nullptr) {
+GVX_HD LcLeg<F> lc_leg_at(const F &pt, const F &mm, const F &r, const uint32_t *n, const gvx_f4 *hyp,
+                          F *sh = nullptr, F *chp = nullptr) {
   using V = lane_t<F>;
-  uint32_t n[2];
-  const F r = lc_reduce(x, n);
   F C, Sh;
   tab_load(hyp, GVX_HYP_N, n, &C, &Sh);
   const TabPoly<V> tp = tab_poly(r, vbc(0.5f, V{}));
@@ -373,16 +370,27 @@ GVX_HD LcLeg<F> lc_leg(const F &pt, const F &mm, const F &x, const gvx_f4 *hyp, 
   l.D = lc_div(q, l.Y);
   return l;
 }
+template <class F>
+GVX_HD LcLeg<F> lc_leg(const F &pt, const F &mm, const F &x, const gvx_f4 *hyp, F *sh = nullptr,
+                       F *chp = nullptr) {
+  uint32_t n[2];
+  const F r = lc_reduce(x, n);
+  return lc_leg_at(pt, mm, r, n, hyp, sh, chp);
+}
 
-// sin and cos of x in [0, 3.5] (x.lo in [0, ulp(x.hi))), absolute error ~2^-46.
-GVX_HD void sincos_lc(const ff &x, const gvx_f4 *sintab, ff *sn, ff *cs) {
-  uint32_t j[1];
-  const ff r = lc_reduce(x, j);
+// sin and cos of x = n 2^-8 + r in [0, 3.5], absolute error ~2^-46.
+GVX_HD void sincos_lc_at(const ff &r, uint32_t n, const gvx_f4 *sintab, ff *sn, ff *cs) {
   ff Sj, Cj;
-  tab_load(sintab, GVX_SIN_N, j, &Sj, &Cj);
+  tab_load(sintab, GVX_SIN_N, &n, &Sj, &Cj);
   const TabPoly<float> tp = tab_poly(r, -0.5f);
   *sn = tab_comb_any(Sj, Cj, r, tp);
   *cs = tab_comb_any(Cj, ff{-Sj.hi, -Sj.lo}, r, tp);
+}
+// The same from x itself (x.lo in [0, ulp(x.hi))).
+GVX_HD void sincos_lc(const ff &x, const gvx_f4 *sintab, ff *sn, ff *cs) {
+  uint32_t j[1];
+  const ff r = lc_reduce(x, j);
+  sincos_lc_at(r, j[0], sintab, sn, cs);
 }
 
 // ---- the pair ------------------------------------------------------------------------------

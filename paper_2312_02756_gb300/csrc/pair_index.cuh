@@ -21,6 +21,26 @@ __device__ __forceinline__ void decode_pair(int64_t k, int64_t n, int64_t &i, in
   j = k - r * (2 * n - r - 1) / 2 + r + 1;
 }
 
+// The same for the sizes that the event kernels stage (n <= 256) in 32-bit integers: the
+// discriminant is an exact float, its approximate root at most one row off.
+__device__ __forceinline__ void decode_pair32(int k, int n, int &i, int &j) {
+  const int b = 2 * n - 1;
+  float root;
+  asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(root) : "f"((float)(b * b - 8 * k)));
+  int r = (int)(((float)b - root) * 0.5f);
+  int start = r * (b - r) >> 1;  // r (2n - r - 1) / 2
+  const int next = start + n - 1 - r;
+  if (start > k) {
+    r--;
+    start -= n - 1 - r;
+  } else if (next <= k) {
+    r++;
+    start = next;
+  }
+  i = r;
+  j = k - start + r + 1;
+}
+
 // The same decoding with a double-precision estimate, for events of any size.
 __device__ __forceinline__ void decode_pair_wide(int64_t k, int64_t n, int64_t &i, int64_t &j) {
   double b = (double)(2 * n - 1);

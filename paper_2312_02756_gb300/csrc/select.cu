@@ -3,62 +3,100 @@
 // RDataFrame-style use of the per-event combinatorics that GenVectorX names as its next target,
 // Sec. 6; the pair mass is that of Sec. 4.1, Fig. 1).  No pair mass is written to memory.
 //
-// CTAs take tiles of kTE consecutive events (grid-stride) and stage them in sub-batches of whole
-// events of at most kNT particles.  Per sub-batch:
-//   (a) one thread per particle: load, cuts, and a block scan of the selection flags that gives
-//       every selected particle its place in a compacted list;
-//   (b) one thread per selected particle: the scale of its event (the largest high word of pt
-//       and |m| over the event's selected particles) and its light-cone terms (pt, Y = E + P,
-//       D = m^2 / Y in float-float at that scale, as the jagged kernel stages them), stored at
-//       its compacted place;
-//       one thread per event: its number of selected pairs, and a block scan of those;
-//   (c) one thread per selected pair (in rounds of kRound): its packed index k in the order of
-//       gvx_event_pair_masses, its mass with the light-cone pair step of the FP64 mass kernels
-//       (mass_lc.cuh; FP64 formulas outside its domain), its histogram slot (shared-memory integer
-//       atomics, so the totals do not depend on the order) and its |m - target| in shared
-//       memory; then one thread per event walks its pairs of the round in order and keeps the
-//       first smallest |m - target| -- exact, and the smaller k on ties.
-// Events of more than kNT particles are handled alone by the whole block, every pair from global
-// memory, with a block reduction of (|m - target|, k).  At the end each CTA adds its histogram
-// to the caller's counts.
+// Each warp takes tiles of up to 32 consecutive events (one per lane) and works through them in
+// batches of its own, synchronised within the warp alone:
+//   (a) batches of whole events of at most kRaw particles: the cuts, one ballot per 32 particles;
+//   (b) of those, runs of whole events with at most kCap selected particles: each selected particle's
+//       raw values go to its place in a compacted list (the place from the ballots), each event
+//       finds its scale (the largest high word of pt and |m| over its selected particles) and its
+//       number of selected pairs, and the list is turned into light-cone terms with fixed-point
+//       angles (event_lc.cuh), 32 at a time;
+//   (c) the selected pairs of the run, 32 at a time: the pair mass, its histogram slot (shared-memory
+//       integer atomics, so the totals do not depend on the order) and its |m - target|, of which
+//       each event keeps the first smallest: the leading words by an integer atomic minimum, the
+//       pairs that reach it (one, but for near ties) by their exact (|m - target|, k) -- exact, and
+//       the smaller packed index k (the order of gvx_event_pair_masses) on ties.
+// What the tiles leave is done after all of a CTA's tiles, in a function of its own (a call inside
+// the tiles costs them spills): pairs outside the float-float domain (near-equal directions, extreme
+// particles), by walking their tiles once more with the elementwise arithmetic for those pairs, and
+// events of more than kCap particles, by the whole block: staged up to kNT particles, else every
+// pair from global memory.  At the end each CTA adds its histogram to the caller's counts.
+//
+// Bound by instruction issue and the latency of its loads (32 M warp instructions at 2^18 events;
+// HBM reads 5% of the time).  2^20 events, 4.2 M selected pairs: 0.188 ms a call, against 0.736 ms
+// for CTA-wide batches of 256 particles, where ten warps in eleven waited at a block barrier; the
+// warps' own batches have none.  Three CTAs of 256 threads per SM: two (0.214 ms) leave too few
+// warps for the load latency, four (64 registers, 0.201 ms) spill and crowd the tables out of L1.
 #include <cuda_runtime.h>
 
-#include <limits.h>
 #include <math.h>
+#include <string.h>
 
 #include "common.cuh"
-#include "mass_lc.cuh"
+#include "event_lc.cuh"
 #include "pair_index.cuh"
-#include "pair_math.cuh"
+#include "pair_raw.cuh"
 
 namespace gvx {
 namespace {
 
-constexpr int kTE = 64;       // events per tile
-constexpr int kNT = 256;      // threads per CTA, and particles per sub-batch
-constexpr int kRound = 512;   // selected pairs evaluated per round
-constexpr int kNoFast = INT_MIN;  // scale marker of a particle outside the float-float domain
-// dynamic shared memory, first part: per compacted particle (pt, Y) and D, eta, phi, scale and
-// original position; per sub-batch particle its scale word and scan value; per round of pairs
-// |m - t|, m and k
-constexpr size_t kDynFixed =
-    (size_t)kNT * (sizeof(float4) + sizeof(float2) + 2 * sizeof(double) + 4 * sizeof(int)) +
-    sizeof(int) + (size_t)kRound * (2 * sizeof(double) + sizeof(long long));
+constexpr int kNT = 256;      // threads per CTA, and particles of an event the block stages
+constexpr int kWarps = kNT / 32;
+constexpr int kRaw = 256;     // particles per batch of a warp (eight ballots)
+constexpr int kCap = 128;     // selected particles per run, and particles of an event a warp takes
+constexpr int kMaxTile = 32;  // events per warp tile, at most
+constexpr unsigned kAll = 0xffffffffu;
 
 struct SArgs {
   Lv p;
   const int64_t *off;
   int64_t n_events, n_particles;
-  double pt_min, eta_max, lo, hi, inv_w, target;
-  int n_bins;
+  long long pt_lo;                       // the cuts (passes)
+  unsigned long long pt_span, eta_end;
+  double lo, hi, inv_w, target;
+  float lo_h, lo_l, inv_f, tol0;  // the float histogram slot (slot_of_ff)
+  int n_bins, tile, turns;        // tile: events per warp tile; turns: a warp's tiles per bit of its rare mask
   unsigned long long *counts;
   int64_t *best_k;
   double *best_m;
   int32_t *status;
 };
 
+// One warp's part of shared memory.
+struct __align__(16) WarpBuf {
+  ffm::EvPart part[kCap];        // by compacted place; tag: position in the batch | event << 8
+  // by event (lane) of the tile: the best pair so far -- the leading word and the bits of its
+  // |m - target|, its mass, its particles' positions in the batch (-1: none)
+  unsigned long long bd[32];
+  double bm[32];
+  uint32_t key[32];
+  int bk[32], own[32];
+  int pp[32], cs[32], n[32];     // by event: first pair and place in the run, selected particles
+  uint32_t scale[32];            // by event: the largest high word of pt and |m|
+};
+
+// The cuts pt >= pt_min and |eta| <= eta_max on the bits of the doubles (an FP64 comparison holds the
+// FP64 pipe like an addition): ordered as signed integers, a double is at least pt_min (and no NaN)
+// when its integer lies in [pt_lo, +inf's]; |eta|'s bits are below eta_end.
+__device__ __forceinline__ long long ordered(double x) {
+  const long long b = __double_as_longlong(x);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
 __device__ __forceinline__ bool passes(double pt, double eta, const SArgs &A) {
-  return pt >= A.pt_min && fabs(eta) <= A.eta_max;
+  return (unsigned long long)(ordered(pt) - A.pt_lo) <= A.pt_span &&
+         ((unsigned long long)__double_as_longlong(eta) & 0x7fffffffffffffffull) < A.eta_end;
+}
+
+// Offsets lo, hi of event e that cannot be right.
+__device__ __forceinline__ bool bad_event(const SArgs &A, int64_t e, int64_t lo, int64_t hi) {
+  return lo < 0 || hi < lo || hi > A.n_particles || (e == 0 && lo != 0) ||
+         (e == A.n_events - 1 && hi != A.n_particles);
+}
+
+// A slot of the CTA's histogram added to the caller's counts.
+__device__ __forceinline__ void flush_slot(const SArgs &A, unsigned *s_hist, int s) {
+  if (s_hist[s]) atomicAdd(A.counts + s, (unsigned long long)s_hist[s]);
+  s_hist[s] = 0u;
 }
 
 // Histogram slot of a mass: 0 below lo, n_bins + 1 at or above hi (and NaN), else 1 + the bin
@@ -72,12 +110,17 @@ __device__ __forceinline__ int slot_of(double m, const SArgs &A) {
   return (int)b + 1;
 }
 
-// The pair mass of two particles given by their raw values (elementwise fast path, FP64 fallback).
-__device__ __forceinline__ double pair_mass_raw(V4<double> x, V4<double> y, const ffm::LcTab &T) {
-  double m;
-  if (!ffm::pair_mass_lc(x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w, T, &m))
-    m = sqrt(pair_terms(make_leg(x), make_leg(y)).m2);
-  return m;
+// The same slot from the mass in float-float at scale 2^(sf's exponent), or -1 where floats do not
+// decide it: t = (m - lo) inv_w is within tol of its exact value (three roundings of 2^-24 of t,
+// and 2^-40 of the range for the low parts left out), so its floor is the bin unless t is within
+// tol of an integer.  The FP64 slot costs six operations of a pipe that a warp instruction holds
+// for ~77 cycles; about one pair in 10^4 needs it (200 bins).
+__device__ __forceinline__ int slot_of_ff(ffm::ff m, float sf, const SArgs &A) {
+  const float x = __fadd_rn(__fsub_rn(__fmul_rn(m.hi, sf), A.lo_h), __fsub_rn(__fmul_rn(m.lo, sf), A.lo_l));
+  float t = __fmul_rn(x, A.inv_f);
+  t = fminf(fmaxf(t, -0.5f), (float)A.n_bins + 0.5f);
+  const float tol = __fmaf_rn(fabsf(t), 4.76837158e-07f, A.tol0);  // 2^-21
+  return fabsf(t - rintf(t)) > tol ? (int)floorf(t) + 1 : -1;
 }
 
 // (d, k) before (d', k'): the smaller |m - target|, then the smaller k; k < 0 is "none".
@@ -85,11 +128,71 @@ __device__ __forceinline__ bool better(double d, long long k, double d0, long lo
   return k >= 0 && (k0 < 0 || d < d0 || (d == d0 && k < k0));
 }
 
+// pt and eta of one particle.
+template <int LP>
+__device__ __forceinline__ void ld_pt_eta(const Lv &v, int64_t i, double &pt, double &eta) {
+  if constexpr (LP == GVX_SOA) {
+    pt = __ldg((const double *)v.c[0] + i);
+    eta = __ldg((const double *)v.c[1] + i);
+  } else {
+    const double2 a = __ldg((const double2 *)v.c[0] + 2 * i);
+    pt = a.x;
+    eta = a.y;
+  }
+}
+
+// A selected particle's place until the leg phase: its raw values (pt, m, eta, phi) and its tag.
+__device__ __forceinline__ void stage_raw(ffm::EvPart &P, const V4<double> &x, uint32_t tag) {
+  *reinterpret_cast<double2 *>(&P.dy) = make_double2(x.x, x.w);
+  *reinterpret_cast<double2 *>(&P.eta) = make_double2(x.y, x.z);
+  P.tag = tag;
+}
+
+// The place from its raw values to light-cone terms at its event's scale word; false outside the
+// float-float domain.
+__device__ __forceinline__ bool stage_leg(ffm::EvPart &P, uint32_t wmax, const ffm::LcTab &T) {
+  const double2 a = *reinterpret_cast<const double2 *>(&P.dy);
+  const double2 b = *reinterpret_cast<const double2 *>(&P.eta);
+  const double pt = a.x, m = a.y, eta = b.x, phi = b.y;
+  const uint32_t hp = ffm::dhi(pt), hm = ffm::dhi(m) & 0x7fffffffu;
+  if (!ffm::lc_in_domain(hp, hm, ffm::dhi(eta) & 0x7fffffffu, ffm::dhi(phi) & 0x7fffffffu, wmax)) {
+    P.scale = 0u;
+    return false;
+  }
+  const uint32_t ew = wmax & 0x7ff00000u, rb = ew - (127u << 20);
+  const ffm::ff ptf = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(pt), rb));
+  const ffm::ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(m), rb));
+  const int64_t ae = ffm::angle_fx(eta);
+  uint32_t n;
+  const ffm::ff r = ffm::fx_half_reduce(2 * ae, &n);
+  const ffm::LcLeg<ffm::ff> L = ffm::lc_leg_at(ptf, mmf, r, &n, T.hyp);
+  P = ffm::EvPart{make_float4(L.D.hi, L.Y.hi, L.D.lo, L.Y.lo), ae, ffm::angle_fx(phi), ptf.hi, ptf.lo, ew, P.tag};
+  return true;
+}
+
+// A pair's mass from its scaled m^2 at the scale field ew; with COUNT its histogram slot counted.
+template <bool COUNT>
+__device__ __forceinline__ double mass_of(ffm::ff m2s, uint32_t ew, const SArgs &A, unsigned *s_hist) {
+  ffm::ff r = {0.0f, 0.0f};
+  double m = 0.0;
+  if (m2s.hi != 0.0f) {
+    r = ffm::lc_sqrt_refined(m2s);
+    r = ffm::fast_two_sum(r.hi, r.lo);
+    m = ffm::lc_to_double_int(r, ew - (127u << 20));
+  }
+  if constexpr (!COUNT) return m;
+  int slot = -1;
+  // 2^(scale) as a float where it is one (2^-100 .. 2^100)
+  if (ew - (923u << 20) <= (200u << 20)) slot = slot_of_ff(r, __uint_as_float((ew - (896u << 20)) << 3), A);
+  if (slot < 0) slot = slot_of(m, A);
+  atomicAdd(&s_hist[slot], 1u);
+  return m;
+}
+
 // One event of more than kNT particles, by the whole block from global memory.
 template <int LP>
-__device__ void big_event_select(const SArgs &A, const ffm::LcTab &T, unsigned *s_hist,
-                                 int64_t pb, int64_t n, double *best_d, long long *best_k,
-                                 double *best_m, double *s_rd, long long *s_rk, double *s_rm) {
+__device__ __noinline__ void big_event_select(const SArgs &A, const ffm::LcTab &T, unsigned *s_hist, int64_t pb,
+                                 int64_t n, double *bd_out, long long *bk_out, double *bm_out) {
   double bd = INFINITY, bm = NAN;
   long long bk = -1;
   const long long npairs = (long long)n * (n - 1) / 2;
@@ -107,220 +210,412 @@ __device__ void big_event_select(const SArgs &A, const ffm::LcTab &T, unsigned *
       bm = m;
     }
   }
-  s_rd[threadIdx.x] = bd;
-  s_rk[threadIdx.x] = bk;
-  s_rm[threadIdx.x] = bm;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int t = 0; t < kNT; t++)
-      if (better(s_rd[t], s_rk[t], bd, bk) || t == 0) {
-        bd = s_rd[t];
-        bk = s_rk[t];
-        bm = s_rm[t];
-      }
-    *best_d = bd;
-    *best_k = bk;
-    *best_m = bm;
-  }
-  __syncthreads();
+  *bd_out = bd;
+  *bk_out = bk;
+  *bm_out = bm;
 }
 
+// One event of more than kCap and at most kNT particles, staged by the whole block: a particle per
+// thread, then its selected pairs over all threads.
 template <int LP>
-__global__ void __launch_bounds__(kNT, 3) pair_select_kernel(SArgs A) {
-  extern __shared__ double s_dyn[];
-  float4 *s_pY = reinterpret_cast<float4 *>(s_dyn);                    // by compacted place
-  float2 *s_D = reinterpret_cast<float2 *>(s_pY + kNT);
-  double *s_eta = reinterpret_cast<double *>(s_D + kNT), *s_phi = s_eta + kNT;
-  double *s_d = s_phi + kNT, *s_m = s_d + kRound;                       // by pair of the round
-  long long *s_k = reinterpret_cast<long long *>(s_m + kRound);
-  int *s_fs = reinterpret_cast<int *>(s_k + kRound), *s_orig = s_fs + kNT;  // by compacted place
-  int *s_ex = s_orig + kNT, *s_cs = s_ex + kNT;  // by particle of the sub-batch (s_cs: kNT + 1)
-  unsigned *s_hist = reinterpret_cast<unsigned *>(s_cs + kNT + 1);
-  __shared__ int64_t s_off[kTE + 1], s_pp[kTE + 1], s_warp[kNT / 32];
-  __shared__ double s_bd[kTE], s_bm[kTE];
-  __shared__ long long s_bk[kTE];
-  __shared__ int s_bad;
-  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) s_hist[s] = 0u;
-  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};  // read through L1
+__device__ __noinline__ void staged_event_select(const SArgs &A, const ffm::LcTab &T, ffm::EvPart *part,
+                                                 unsigned *s_hist, int64_t pb, int n, double *bd_out,
+                                                 long long *bk_out, double *bm_out) {
+  __shared__ int64_t s_warp[kWarps];
+  __shared__ unsigned s_scale;
+  const int k = threadIdx.x;
+  V4<double> x = {0.0, 0.0, 0.0, 0.0};
+  const bool in = k < n;
+  if (in) x = ld4<double, LP>(A.p, pb + k);
+  const bool pass = in && passes(x.x, x.y, A);
+  if (k == 0) s_scale = 0u;
+  int64_t nsel;
+  const int c = (int)block_excl_scan<kNT>(pass ? 1 : 0, s_warp, &nsel);  // ends synchronised
+  if (pass) {
+    stage_raw(part[c], x, (uint32_t)k);
+    atomicMax(&s_scale, ffm::umax32(ffm::dhi(x.x), ffm::dhi(x.w) & 0x7fffffffu));
+  }
+  __syncthreads();
+  if (k < (int)nsel) stage_leg(part[k], s_scale, T);
+  __syncthreads();
+  const int ns = (int)nsel, total = ns * (ns - 1) / 2;
+  double bd = INFINITY, bm = NAN;
+  long long bk = -1;
+  for (int q = k; q < total; q += kNT) {
+    int i, j;
+    decode_pair32(q, ns, i, j);
+    const ffm::EvPart &a = part[i], &b = part[j];
+    const int oi = (int)a.tag, oj = (int)b.tag;
+    ffm::ff m2s;
+    double m;
+    if (a.scale != 0u && b.scale != 0u && ffm::ev_pair_m2(a, b, T, &m2s)) {
+      m = mass_of<true>(m2s, a.scale, A, s_hist);
+    } else {
+      m = pair_mass_at<LP>(A.p.c[0], A.p.c[1], A.p.c[2], A.p.c[3], pb + oi, pb + oj);
+      atomicAdd(&s_hist[slot_of(m, A)], 1u);
+    }
+    double d = fabs(m - A.target);
+    if (q == 0 && isnan(d)) d = -1.0;  // a first pair without a distance is never replaced
+    const long long kk = oi * n - oi * (oi + 1) / 2 + (oj - oi - 1);
+    if (better(d, kk, bd, bk)) {
+      bd = d;
+      bk = kk;
+      bm = m;
+    }
+  }
+  *bd_out = bd;
+  *bk_out = bk;
+  *bm_out = bm;
+}
 
-  const int64_t n_tiles = (A.n_events + kTE - 1) / kTE;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t e0 = tile * kTE;
-    const int ne = (int)(A.n_events - e0 < kTE ? A.n_events - e0 : kTE);
-    __syncthreads();  // the previous tile is done with the shared arrays
-    if (threadIdx.x == 0) s_bad = 0;
-    if (threadIdx.x <= ne) s_off[threadIdx.x] = A.off[e0 + threadIdx.x];
-    if (threadIdx.x < ne) {
-      s_bd[threadIdx.x] = INFINITY;
-      s_bk[threadIdx.x] = -1;
-      s_bm[threadIdx.x] = NAN;
-    }
-    __syncthreads();
-    if (threadIdx.x < ne) {
-      const int64_t a = s_off[threadIdx.x], b = s_off[threadIdx.x + 1];
-      bool bad = a < 0 || b < a || b > A.n_particles;
-      if (e0 + threadIdx.x == 0 && a != 0) bad = true;
-      if (e0 + threadIdx.x == A.n_events - 1 && b != A.n_particles) bad = true;
-      if (bad) s_bad = 1;
-    }
-    __syncthreads();
-    if (s_bad) {  // nothing of the tile is read; its events report no candidate
-      if (threadIdx.x == 0) raise_status(A.status, GVX_ERR_OFFSETS);
-      if (threadIdx.x < ne) {
-        if (A.best_k) A.best_k[e0 + threadIdx.x] = -1;
-        if (A.best_m) A.best_m[e0 + threadIdx.x] = NAN;
+// The particles of pair q of a run: places ci, cj and the event (lane) e.
+__device__ __forceinline__ void pair_places(const WarpBuf &W, int q, int &e, int &ci, int &cj) {
+  e = 0;  // the last event whose first pair is <= q
+#pragma unroll
+  for (int step = 16; step > 0; step >>= 1)
+    if (W.pp[e + step] <= q) e += step;
+  int i, j;
+  decode_pair32(q - W.pp[e], W.n[e], i, j);
+  ci = W.cs[e] + i;
+  cj = W.cs[e] + j;
+}
+
+// Pairs of mass m and particle positions k (row-major order as an integer) offered to their events'
+// best, by the whole warp; first: the event's first pair, which stays if it has no distance (NaN).
+__device__ __forceinline__ void offer(WarpBuf &W, bool valid, int e, double m, int k, bool first,
+                                      const SArgs &A) {
+  const int lane = threadIdx.x & 31;
+  // distances are non-negative: their bits order them, NaN last
+  unsigned long long d = (unsigned long long)__double_as_longlong(fabs(m - A.target));
+  if (first && d > 0x7ff0000000000000ull) d = 0ull;
+  const uint32_t key = (uint32_t)(d >> 32);
+  if (valid) atomicMin(&W.key[e], key);
+  __syncwarp();
+  bool cand = valid && key == W.key[e];
+  while (__any_sync(kAll, cand)) {
+    if (cand) W.own[e] = lane;
+    __syncwarp();
+    if (cand && W.own[e] == lane) {
+      const unsigned long long d0 = W.bd[e];
+      const int k0 = W.bk[e];
+      if (k0 < 0 || d < d0 || (d == d0 && k < k0)) {
+        W.bd[e] = d;
+        W.bm[e] = m;
+        W.bk[e] = k;
       }
-      continue;
+      cand = false;
     }
+    __syncwarp();
+  }
+}
+
+// One warp tile: events e0 .. e0 + ne - 1 (ne <= 32), lane l having event e0 + l with particles
+// lo .. hi - 1.  Returns kLarge when it left an event to the block, kRare when it left a pair to a
+// second walk.  RARE: that walk, which counts the pairs left and forms the best ones anew.
+constexpr int kLarge = 1, kRare = 2;
+
+template <int LP, bool RARE>
+__device__ __forceinline__ int warp_tile(const SArgs &A, const ffm::LcTab &T, WarpBuf &W,
+                                          unsigned *s_hist, int64_t e0, int ne, int64_t lo, int64_t hi) {
+  const int lane = threadIdx.x & 31;
+  const unsigned below = (1u << lane) - 1u;
+  W.key[lane] = 0xffffffffu;
+  W.bk[lane] = -1;
+  W.bm[lane] = NAN;
+  int left = 0;
+  if (__any_sync(kAll, lane < ne && bad_event(A, e0 + lane, lo, hi))) {
+    // nothing of the tile is read; its events report no candidate
+    if (lane == 0) raise_status(A.status, GVX_ERR_OFFSETS);
+  } else {
     int sb = 0;
     while (sb < ne) {
-      const int64_t pb = s_off[sb];
-      const bool fits =
-          threadIdx.x >= sb && threadIdx.x < ne && s_off[threadIdx.x + 1] - pb <= kNT;
-      const int sbe = sb + __syncthreads_count(fits);
-      if (sbe == sb) {  // one event larger than a sub-batch
-        big_event_select<LP>(A, T, s_hist, pb, s_off[sb + 1] - pb, &s_bd[sb], &s_bk[sb],
-                             &s_bm[sb], s_d, s_k, s_m);
+      // (a) a batch of whole events: at most kRaw particles, none of more than kCap
+      const int64_t pb = __shfl_sync(kAll, lo, sb);
+      const unsigned ok =
+          __ballot_sync(kAll, lane >= sb && lane < ne && hi - lo <= kCap && hi - pb <= kRaw) >> sb;
+      const int take = ok == kAll ? 32 : __ffs((int)~ok) - 1;  // the leading ones that fit
+      if (take == 0) {  // an event for the block
+        left |= kLarge;
         sb++;
         continue;
       }
-      const int np = (int)(s_off[sbe] - pb), nev = sbe - sb;
-      const int k = threadIdx.x;
-      // (a) cuts and compaction
-      V4<double> x = {0.0, 0.0, 0.0, 0.0};
-      bool pass = false;
-      if (k < np) {
-        x = ld4<double, LP>(A.p, pb + k);
-        pass = passes(x.x, x.y, A);
-        s_ex[k] = pass ? (int)ffm::umax32(ffm::dhi(x.x), ffm::dhi(x.w) & 0x7fffffffu) : 0;
-      }
-      int64_t nsel;
-      const int c = (int)block_excl_scan<kNT>(pass ? 1 : 0, s_warp, &nsel);  // ends synchronised
-      if (k < np) s_cs[k] = c;
-      if (k == 0) s_cs[np] = (int)nsel;
-      // (b) legs of the selected particles; selected pairs per event
-      if (pass) {
-        int e = sb, hi = sbe - 1;  // the particle's event: the last e with s_off[e] <= pb + k
-        while (e < hi) {
-          const int mid = (e + hi + 1) >> 1;
-          if (s_off[mid] <= pb + k) e = mid;
-          else hi = mid - 1;
+      const int sbe = sb + take;
+      const int np = (int)(__shfl_sync(kAll, hi, sbe - 1) - pb);
+      unsigned word = 0;  // lane r: the selection bits of particles 32 r .. 32 r + 31
+      for (int r = 0; r < np; r += 128) {
+        double pt[4], eta[4];
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          pt[u] = eta[u] = NAN;  // fails the cuts
+          if (r + 32 * u + lane < np) ld_pt_eta<LP>(A.p, pb + r + 32 * u + lane, pt[u], eta[u]);
         }
-        uint32_t wmax = 0;  // the event's scale word over its selected particles
-        for (int t = (int)(s_off[e] - pb); t < (int)(s_off[e + 1] - pb); t++)
-          wmax = ffm::umax32((uint32_t)s_ex[t], wmax);
-        // the domain of the elementwise fast path (mass_lc.cuh), at the event's scale
-        const uint32_t ew = wmax & 0x7ff00000u;
-        const uint32_t hp = ffm::dhi(x.x), hm = ffm::dhi(x.w) & 0x7fffffffu;
-        const uint32_t he = ffm::dhi(x.y) & 0x7fffffffu, hf = ffm::dhi(x.z) & 0x7fffffffu;
-        int sc = kNoFast;
-        if (wmax - (200u << 20) < (1700u << 20) &&
-            ffm::umin32(hp - 0x100000u, hm - 0x100000u) >= ew - (41u << 20) &&
-            ffm::umax32(hp, hm) >= 0x100000u && he < 0x40200000u && hf < 0x400C0000u) {
-          const uint32_t rb = ew - (127u << 20);
-          const ffm::ff ptf = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(x.x), rb));
-          const ffm::ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(x.w), rb));
-          const ffm::ff xe = ffm::cvt1(ffm::cvt_parts_normal(ffm::umax32(he, 0x3E100000u),
-                                                             ffm::dlo(x.y), ffm::kRebaseOne));
-          const ffm::LcLeg<ffm::ff> L = ffm::lc_leg(ptf, mmf, xe, T.hyp);
-          s_pY[c] = make_float4(ptf.hi, ptf.lo, L.Y.hi, L.Y.lo);
-          s_D[c] = make_float2(L.D.hi, L.D.lo);
-          sc = (int)ew;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          const unsigned b = __ballot_sync(kAll, passes(pt[u], eta[u], A));
+          if (lane == r / 32 + u) word = b;
         }
-        s_fs[c] = sc;
-        s_orig[c] = k;
-        s_eta[c] = x.y;
-        s_phi[c] = x.z;
       }
-      __syncthreads();  // s_cs complete
-      int64_t npairs_ev = 0;
-      if (threadIdx.x < nev) {
-        const int st = (int)(s_off[sb + threadIdx.x] - pb), en = (int)(s_off[sb + threadIdx.x + 1] - pb);
-        const int64_t ns = s_cs[en] - s_cs[st];
-        npairs_ev = ns * (ns - 1) / 2;
+      // selected particles before position 32 lane, then before each event's first particle and
+      // before the one after its last
+      int pre = __popc(word);
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const int y = __shfl_up_sync(kAll, pre, o);
+        if (lane >= o) pre += y;
       }
-      int64_t total;
-      const int64_t pex = block_excl_scan<kNT>(npairs_ev, s_warp, &total);  // ends synchronised
-      if (threadIdx.x < nev) s_pp[threadIdx.x] = pex;
-      if (threadIdx.x == 0) s_pp[nev] = total;
-      __syncthreads();
-      // (c) the selected pairs, in rounds
-      for (int64_t r0 = 0; r0 < total; r0 += kRound) {
-        const int64_t r1 = total - r0 < kRound ? total : r0 + kRound;
-        for (int64_t q = r0 + threadIdx.x; q < r1; q += kNT) {
-          int e = 0, hi = nev - 1;  // the pair's event within the sub-batch
-          while (e < hi) {
-            const int mid = (e + hi + 1) >> 1;
-            if (s_pp[mid] <= q) e = mid;
-            else hi = mid - 1;
-          }
-          const int st = (int)(s_off[sb + e] - pb);
-          const int64_t n = s_off[sb + e + 1] - s_off[sb + e];
-          const int64_t ns = s_cs[st + (int)n] - s_cs[st];
-          int64_t a, b;
-          decode_pair(q - s_pp[e], ns, a, b);
-          const int ci = s_cs[st] + (int)a, cj = s_cs[st] + (int)b;
-          const int64_t i = s_orig[ci] - st, j = s_orig[cj] - st;  // positions in the event
-          double m;
-          bool done = false;
-          const int sc = s_fs[ci];
-          if (sc != kNoFast && s_fs[cj] != kNoFast) {
-            ffm::ff S, m2s;
-            const bool oks = ffm::lc_pair_S(s_eta[ci], s_eta[cj], s_phi[ci], s_phi[cj], T, &S);
-            const float4 a4 = s_pY[ci], b4 = s_pY[cj];
-            const float2 da = s_D[ci], db = s_D[cj];
-            if (ffm::lc_pair_m2(ffm::ff{a4.x, a4.y}, ffm::ff{b4.x, b4.y}, ffm::ff{a4.z, a4.w},
-                                ffm::ff{b4.z, b4.w}, ffm::ff{da.x, da.y}, ffm::ff{db.x, db.y}, S,
-                                &m2s) && oks) {
-              m = ffm::lc_mass_out_int(m2s, (uint32_t)sc);
-              done = true;
+      pre -= __popc(word);
+      const bool mine = lane >= sb && lane < sbe;
+      const int s0 = mine ? (int)(lo - pb) : np, s1 = mine ? (int)(hi - pb) : np;
+      const int w0 = __shfl_sync(kAll, (int)word, s0 >> 5), f0 = __shfl_sync(kAll, pre, s0 >> 5);
+      const int w1 = __shfl_sync(kAll, (int)word, s1 >> 5), f1 = __shfl_sync(kAll, pre, s1 >> 5);
+      const int c0 = f0 + __popc((unsigned)w0 & ((1u << (s0 & 31)) - 1u));
+      const int c1 = f1 + __popc((unsigned)w1 & ((1u << (s1 & 31)) - 1u));
+      // (b), (c) runs of whole events with at most kCap selected particles
+      int rb = sb;
+      while (rb < sbe) {
+        const int cbase = __shfl_sync(kAll, c0, rb);
+        const int re = rb + __popc(__ballot_sync(kAll, lane >= rb && lane < sbe && c1 - cbase <= kCap));
+        const int ns = __shfl_sync(kAll, c1, re - 1) - cbase;  // re > rb: an event has at most kCap
+        const bool run = lane >= rb && lane < re;
+        const int nse = run ? c1 - c0 : 0;
+        int pp = nse * (nse - 1) / 2;
+        const int npairs = pp;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int y = __shfl_up_sync(kAll, pp, o);
+          if (lane >= o) pp += y;
+        }
+        const int total = __shfl_sync(kAll, pp, 31);
+        if (total > 0) {
+          W.pp[lane] = pp - npairs;
+          W.cs[lane] = c0 - cbase;
+          W.n[lane] = nse;
+          // the selected particles of the run, each at its place
+          const int first = (int)(__shfl_sync(kAll, lo, rb) - pb);
+          const int last = (int)(__shfl_sync(kAll, hi, re - 1) - pb);
+          for (int r = first & ~31; r < last; r += 32) {
+            const unsigned b = (unsigned)__shfl_sync(kAll, (int)word, r >> 5);
+            const int f = __shfl_sync(kAll, pre, r >> 5) - cbase;
+            const int i = r + lane;
+            if (((b >> lane) & 1u) && i >= first && i < last) {
+              stage_raw(W.part[f + __popc(b & below)], ld4c<LP>(A.p, pb + i), (uint32_t)i);
             }
           }
-          if (!done) m = pair_mass_raw(ld4c<LP>(A.p, pb + st + i), ld4c<LP>(A.p, pb + st + j), T);
-          atomicAdd(&s_hist[slot_of(m, A)], 1u);
-          s_d[q - r0] = fabs(m - A.target);
-          s_m[q - r0] = m;
-          s_k[q - r0] = i * n - i * (i + 1) / 2 + (j - i - 1);
-        }
-        __syncthreads();
-        if (threadIdx.x < nev) {  // each event's pairs of the round, in order
-          const int e = threadIdx.x;
-          const int64_t q0 = s_pp[e] > r0 ? s_pp[e] : r0, q1 = s_pp[e + 1] < r1 ? s_pp[e + 1] : r1;
-          double bd = s_bd[sb + e], bm = s_bm[sb + e];
-          long long bk = s_bk[sb + e];
-          for (int64_t q = q0; q < q1; q++)
-            if (better(s_d[q - r0], s_k[q - r0], bd, bk)) {
-              bd = s_d[q - r0];
-              bk = s_k[q - r0];
-              bm = s_m[q - r0];
+          __syncwarp();
+          if (run) {  // the event's scale; its particles learn their event
+            uint32_t wmax = 0;
+            for (int c = c0 - cbase; c < c1 - cbase; c++) {
+              const double2 a = *reinterpret_cast<const double2 *>(&W.part[c].dy);
+              wmax = ffm::umax32(ffm::umax32(ffm::dhi(a.x), ffm::dhi(a.y) & 0x7fffffffu), wmax);
+              W.part[c].tag |= (uint32_t)lane << 8;
             }
-          s_bd[sb + e] = bd;
-          s_bk[sb + e] = bk;
-          s_bm[sb + e] = bm;
+            W.scale[lane] = wmax;
+          }
+          __syncwarp();
+          bool extreme = false;
+          for (int c = lane; c < ns; c += 32)
+            extreme |= !stage_leg(W.part[c], W.scale[W.part[c].tag >> 8], T);
+          extreme = __any_sync(kAll, extreme);  // and the staged places are visible to the warp
+          bool rare = false;
+          for (int r0 = 0; r0 < total; r0 += 32) {
+            const int q = r0 + lane;
+            int e = 0, k = 0;
+            bool offered = false, fst = false;
+            double m = 0.0;
+            if (q < total) {
+              int ci, cj;
+              pair_places(W, q, e, ci, cj);
+              const ffm::EvPart &a = W.part[ci], &b = W.part[cj];
+              const int oi = a.tag & 0xff, oj = b.tag & 0xff;
+              ffm::ff m2s;
+              const bool fast = !(extreme && (a.scale == 0u || b.scale == 0u)) && ffm::ev_pair_m2(a, b, T, &m2s);
+              if (fast) m = mass_of<!RARE>(m2s, a.scale, A, s_hist);
+              if constexpr (RARE) {
+                if (!fast) {
+                  m = pair_mass_at<LP>(A.p.c[0], A.p.c[1], A.p.c[2], A.p.c[3], pb + oi, pb + oj);
+                  atomicAdd(&s_hist[slot_of(m, A)], 1u);
+                }
+              }
+              offered = RARE || fast;
+              rare |= !fast;
+              k = oi << 8 | oj;
+              fst = q == W.pp[e];
+            }
+            offer(W, offered, e, m, k, fst, A);
+          }
+          if (__any_sync(kAll, rare)) left |= kRare;
+          __syncwarp();  // before the next run's particles
+          if (run && W.bk[lane] >= 0) {  // positions in the batch -> the packed index in the event
+            const int n = (int)(hi - lo), k = W.bk[lane];
+            const int i = (k >> 8) - (int)(lo - pb), j = (k & 0xff) - (int)(lo - pb);
+            W.bk[lane] = i * n - i * (i + 1) / 2 + (j - i - 1);
+          }
         }
-        __syncthreads();
+        rb = re;
       }
       sb = sbe;
     }
-    __syncthreads();
-    if (threadIdx.x < ne) {
-      if (A.best_k) A.best_k[e0 + threadIdx.x] = s_bk[threadIdx.x];
-      if (A.best_m) A.best_m[e0 + threadIdx.x] = s_bk[threadIdx.x] >= 0 ? s_bm[threadIdx.x] : NAN;
-    }
   }
-  __syncthreads();
-  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT)
-    if (s_hist[s]) atomicAdd(A.counts + s, (unsigned long long)s_hist[s]);
+  __syncwarp();
+  if (lane < ne) {
+    if (A.best_k) A.best_k[e0 + lane] = W.bk[lane];
+    if (A.best_m) A.best_m[e0 + lane] = W.bm[lane];
+  }
+  __syncwarp();
+  return left;
+}
+
+// Asks L2 for the lines of particles lo .. hi - 1 (nothing for a range that cannot be right).
+template <int LP>
+__device__ __forceinline__ void prefetch_particles(const SArgs &A, int64_t lo, int64_t hi) {
+  if (lo < 0 || hi <= lo || hi > A.n_particles || hi - lo > 1024) return;
+  const int bytes = (int)(hi - lo) * (LP == GVX_SOA ? 8 : 32);
+#pragma unroll
+  for (int c = 0; c < (LP == GVX_SOA ? 4 : 1); c++) {
+    const char *p = (const char *)A.p.c[c] + lo * (LP == GVX_SOA ? 8 : 32);
+    for (int o = 128 * (threadIdx.x & 31); o < bytes; o += 128 * 32)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(p + o));
+  }
+}
+
+// Events of warp tile t.
+__device__ __forceinline__ int events_of(const SArgs &A, int64_t t) {
+  const int64_t rest = A.n_events - t * A.tile;
+  return (int)(rest < A.tile ? rest : A.tile);
+}
+
+// What the tiles of a CTA left: rare, per warp, the tiles with pairs to walk again; then the events
+// of more than kCap particles, by the whole block.
+template <int LP>
+__device__ __noinline__ void finish_tiles(const SArgs &A, unsigned char *s_dyn, unsigned *s_hist,
+                                          int64_t n_tiles, unsigned long long rare) {
+  __shared__ int64_t s_off[kWarps][kMaxTile + 1];
+  __shared__ int s_ne[kWarps];
+  __shared__ double s_rd[kNT], s_rm[kNT];
+  __shared__ long long s_rk[kNT];
+  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  bool large = false;
+  int64_t turn = 0;
+  for (int64_t t0 = (int64_t)blockIdx.x * kWarps; t0 < n_tiles; t0 += (int64_t)gridDim.x * kWarps, turn++) {
+    const int64_t t = t0 + warp;
+    const int ne = t < n_tiles ? events_of(A, t) : 0;
+    int64_t lo = 0, hi = 0;
+    if (lane < ne) {
+      lo = A.off[t * A.tile + lane];
+      hi = A.off[t * A.tile + lane + 1];
+    }
+    const bool bad = __any_sync(kAll, lane < ne && bad_event(A, t * A.tile + lane, lo, hi));
+    if (!bad && ((rare >> (turn / A.turns)) & 1ull))
+      warp_tile<LP, true>(A, T, reinterpret_cast<WarpBuf *>(s_dyn)[warp], s_hist, t * A.tile, ne, lo, hi);
+    large |= !bad && lane < ne && hi - lo > kCap;
+  }
+  if (!__syncthreads_or(large)) return;
+  ffm::EvPart *part = reinterpret_cast<ffm::EvPart *>(s_dyn);
+  static_assert(sizeof(WarpBuf) * kWarps >= kNT * sizeof(ffm::EvPart), "an event staged by the block");
+  for (int64_t t0 = (int64_t)blockIdx.x * kWarps; t0 < n_tiles; t0 += (int64_t)gridDim.x * kWarps) {
+    const int64_t t = t0 + warp;
+    const int ne = t < n_tiles ? events_of(A, t) : 0;
+    bool bad = false;
+    if (lane < ne) {
+      const int64_t lo = A.off[t * A.tile + lane], hi = A.off[t * A.tile + lane + 1];
+      bad = bad_event(A, t * A.tile + lane, lo, hi);
+      s_off[warp][lane] = lo;
+      if (lane == ne - 1) s_off[warp][ne] = hi;
+    }
+    bad = __any_sync(kAll, bad);
+    if (lane == 0) s_ne[warp] = bad ? 0 : ne;
+    __syncthreads();
+    for (int w = 0; w < kWarps; w++) {
+      for (int e = 0; e < s_ne[w]; e++) {
+        const int64_t pb = s_off[w][e], n = s_off[w][e + 1] - pb, ev = (t0 + w) * A.tile + e;
+        if (n <= kCap) continue;
+        if (n <= kNT)
+          staged_event_select<LP>(A, T, part, s_hist, pb, (int)n, &s_rd[threadIdx.x], &s_rk[threadIdx.x],
+                                  &s_rm[threadIdx.x]);
+        else
+          big_event_select<LP>(A, T, s_hist, pb, n, &s_rd[threadIdx.x], &s_rk[threadIdx.x], &s_rm[threadIdx.x]);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          double bd = s_rd[0], bm = s_rm[0];
+          long long bk = s_rk[0];
+          for (int u = 1; u < kNT; u++)
+            if (better(s_rd[u], s_rk[u], bd, bk)) {
+              bd = s_rd[u];
+              bk = s_rk[u];
+              bm = s_rm[u];
+            }
+          if (A.best_k) A.best_k[ev] = bk;
+          if (A.best_m) A.best_m[ev] = bk >= 0 ? bm : NAN;
+        }
+        __syncthreads();
+        if (n > kNT) {  // so that no slot of the CTA's counts can pass 2^32
+          for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) flush_slot(A, s_hist, s);
+          __syncthreads();
+        }
+      }
+    }
+    __syncthreads();  // before the next tiles' offsets
+  }
 }
 
 template <int LP>
-cudaError_t launch_l(const SArgs &A, cudaStream_t s) {
+__global__ void __launch_bounds__(kNT, 3) pair_select_kernel(const __grid_constant__ SArgs A) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  WarpBuf *bufs = reinterpret_cast<WarpBuf *>(s_dyn);
+  unsigned *s_hist = reinterpret_cast<unsigned *>(bufs + kWarps);
+  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) s_hist[s] = 0u;
+  __syncthreads();
+  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};  // read through L1
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int64_t n_tiles = (A.n_events + A.tile - 1) / A.tile;
+  // a tile's offsets are loaded one tile ahead, and its particles' lines asked for then
+  const auto offsets_of = [&](int64_t t, int64_t &lo, int64_t &hi) {
+    lo = hi = 0;
+    if (t < n_tiles && lane < events_of(A, t)) {
+      lo = A.off[t * A.tile + lane];
+      hi = A.off[t * A.tile + lane + 1];
+    }
+  };
+  const int64_t step = (int64_t)gridDim.x * kWarps;
+  int64_t t = (int64_t)blockIdx.x * kWarps + warp, lo, hi;
+  bool large = false;
+  unsigned long long rare = 0;  // the warp's tiles to walk again, one bit for 1/64 of them
+  offsets_of(t, lo, hi);
+  for (int64_t turn = 0; t < n_tiles; t += step, turn++) {
+    int64_t lo1, hi1;
+    offsets_of(t + step, lo1, hi1);
+    if (t + step < n_tiles)
+      prefetch_particles<LP>(A, __shfl_sync(kAll, lo1, 0), __shfl_sync(kAll, hi1, events_of(A, t + step) - 1));
+    const int left = warp_tile<LP, false>(A, T, bufs[warp], s_hist, t * A.tile, events_of(A, t), lo, hi);
+    large |= (left & kLarge) != 0;
+    if (left & kRare) rare |= 1ull << (turn / A.turns);
+    lo = lo1;
+    hi = hi1;
+  }
+  if (__syncthreads_or(large || rare != 0)) finish_tiles<LP>(A, s_dyn, s_hist, n_tiles, rare);
+  __syncthreads();
+  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) flush_slot(A, s_hist, s);
+}
+
+template <int LP>
+cudaError_t launch_l(SArgs A, cudaStream_t s) {
   constexpr auto k = pair_select_kernel<LP>;
-  const size_t smem = kDynFixed + (size_t)(A.n_bins + 2) * sizeof(unsigned);
+  const size_t smem = kWarps * sizeof(WarpBuf) + (size_t)(A.n_bins + 2) * sizeof(unsigned);
   cudaError_t err = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
-  const int64_t n_tiles = (A.n_events + kTE - 1) / kTE;
-  k<<<balanced_grid_of<k>(kNT, smem, n_tiles, 1), kNT, smem, s>>>(A);
+  // resident CTAs; a small call takes smaller tiles, so that its events reach all of their warps
+  int per_sm = 0;
+  err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kNT, smem);
+  if (err != cudaSuccess) return err;
+  const int64_t warps = (int64_t)num_sms() * (per_sm < 1 ? 1 : per_sm) * kWarps;
+  const int64_t want = (A.n_events + warps - 1) / warps;
+  A.tile = (int)(want < kMaxTile ? want : kMaxTile);
+  const int64_t n_tiles = (A.n_events + A.tile - 1) / A.tile;
+  const int64_t need = (n_tiles + kWarps - 1) / kWarps, cap = warps / kWarps;
+  const int64_t grid = need < cap ? need : cap;
+  A.turns = (int)((n_tiles + 64 * grid * kWarps - 1) / (64 * grid * kWarps));
+  k<<<(unsigned)grid, kNT, smem, s>>>(A);
   return cudaGetLastError();
 }
 
@@ -335,13 +630,30 @@ cudaError_t launch_pair_select(const Lv &p, const int64_t *off, int64_t n_events
   A.off = off;
   A.n_events = n_events;
   A.n_particles = n_particles;
-  A.pt_min = pt_min;
-  A.eta_max = eta_max;
+  // the cuts on ordered integers: -0 passes a threshold of 0, nothing passes a NaN
+  const auto bits = [](double x) {
+    long long b;
+    memcpy(&b, &x, sizeof b);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+  };
+  const long long inf = bits(INFINITY);
+  A.pt_lo = pt_min == 0.0 ? bits(-0.0) : bits(pt_min);
+  A.pt_span = (unsigned long long)inf - (unsigned long long)A.pt_lo;
+  A.eta_end = eta_max >= 0.0 ? (unsigned long long)bits(fabs(eta_max)) + 1ull : 0ull;
+  if (!(pt_min <= INFINITY)) A.eta_end = 0ull;
   A.lo = lo;
   A.hi = hi;
   A.inv_w = (double)n_bins / (hi - lo);
   A.target = target;
   A.n_bins = n_bins;
+  // the float slot: lo in two floats, 1/width, and the absolute part of its error; a range or width
+  // outside the floats leaves every pair to the FP64 slot (an infinite tolerance)
+  const double inv_abs = fabs(A.inv_w), reach = fabs(lo) + fabs(hi);
+  const bool fits = inv_abs > 1e-30 && inv_abs < 1e30 && reach < 1e30;
+  A.lo_h = fits ? (float)lo : 0.0f;
+  A.lo_l = fits ? (float)(lo - (double)A.lo_h) : 0.0f;
+  A.inv_f = fits ? (float)A.inv_w : 0.0f;
+  A.tol0 = fits ? (float)(reach * A.inv_w * 0x1p-40) + 0x1p-40f : INFINITY;
   A.counts = reinterpret_cast<unsigned long long *>(counts);
   A.best_k = best_k;
   A.best_m = best_m;
