@@ -5,41 +5,47 @@
 // Work unit: a tile of TE consecutive events.  CTAs take tiles in increasing order from an
 // atomic counter and stay resident until the tiles run out.  Per tile:
 //   1. load and validate offsets[e0 .. e0+TE];  n_e(n_e-1)/2 pairs per event, block scan;
-//   2. decoupled look-back over the tile descriptors for the number of pairs before the tile
-//      (bounded wait: a predecessor that never publishes makes the CTA record GVX_ERR_TIMEOUT
-//      and go on);  write pair_offsets;
-//   3. stage the tile's particles in shared memory in sub-batches of at most kCP particles:
-//      per-particle terms once per particle (one thread each, which also finds its event's
-//      scale) -- the float-float light-cone terms of the leg (pt, Y = E + P, D = m^2 / Y, scaled
-//      by the event's power of two, bit for bit a lane of the elementwise FP64 kernel's legs) and
-//      the Cartesian components for the sums, in float-float -- then, after one barrier, the
-//      event sums (one thread per event and component, float-float at the event's scale and one
-//      conversion per sum) and the pair masses (one thread per pair over the flattened pair range
-//      of the sub-batch, coalesced stores) with the elementwise kernel's pair arithmetic
-//      (mass_lc.cuh: lc_pair_m2; the output assembled by integer operations, so that a pair
-//      costs two FP64 operations), falling back to FP64 for pairs outside its domain;
-//   4. an event with more than kCP particles is handled alone, straight from global memory.
+//   2. decoupled look-back over the tile descriptors, 32 at a time, for the number of pairs before
+//      the tile (bounded wait: a predecessor that never publishes makes the CTA record
+//      GVX_ERR_TIMEOUT and go on);  write pair_offsets;
+//   3. the tile's events in batches of whole events of at most kCapW particles, each batch by one
+//      warp with its own part of shared memory and no block barrier: per particle once, the
+//      float-float light-cone terms of its leg (pt, Y = E + P, D = m^2 / Y at its event's power of
+//      two), its angles in fixed point (event_lc.cuh) and its Cartesian components in float-float;
+//      then the event sums (two components per lane as the lanes of paired FP32 instructions, the
+//      event's particles split over two lanes) and the pair masses, one lane per pair over the
+//      batch's flattened pairs, coalesced stores.  A pair finds its particles from a bit mask of
+//      the rows' first pairs (a row: one particle with its later partners): one popcount and one
+//      row record instead of a search for the event and a decoding of the index.
+//   4. What the batches leave is done after them, in a function of its own at the end of the tile (a
+//      call inside the batches costs them spills): pairs outside the float-float domain (near-equal
+//      directions, extreme particles), by walking the tile's batches once more and giving those
+//      pairs the elementwise arithmetic; and events with more than kCapW particles, by the whole CTA,
+//      staged the same way up to kCP particles, straight from global memory beyond.
 // Tile descriptors are 64-bit words: 2 flag bits (aggregate / inclusive prefix) + 62-bit value.
+//
+// Bound by issue and the shared-memory/L1 data pipe together (430 warp instructions and 115 data
+// wavefronts per 32 pairs, of which the two table gathers take about 40).  2^20 events, 33.5 M
+// pairs: 0.582 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
+// and a search per pair (620 instructions per 32 pairs, FP64 pipe 35% busy).  Six CTAs of 128
+// threads per SM (80 registers): eight (64 registers, 0.623 ms) leave the tables too little L1.
+// Tiles of 64 events on 128 threads: 0.615 ms; 256 on 256: 0.587 ms.
 #include <cuda_runtime.h>
 
 #include <type_traits>
 
-#include <limits.h>
-
 #include "common.cuh"
-#include "mass_lc.cuh"
+#include "event_lc.cuh"
 #include "pair_index.cuh"
-#include "pair_math.cuh"
+#include "pair_raw.cuh"
 
 namespace gvx {
 namespace {
 
-// particles staged in shared memory per sub-batch
-constexpr int kCP = 224;
-// per particle: eta, phi, px, py, pz, E (doubles), pt, Y, D (float pairs), the particle's
-// largest high word of pt and |m|, and its event's scale field or kNoFast (ints)
-constexpr size_t kDynSmem = (size_t)kCP * (6 * sizeof(double) + 3 * sizeof(float2) + 2 * sizeof(int));
-constexpr int kNoFast = INT_MIN;  // scale marker of a particle outside the float-float domain
+constexpr int kCapW = 64;  // particles per warp batch
+constexpr int kCP = 224;   // particles of an event that the CTA stages
+constexpr int kRows = kCapW * (kCapW - 1) / 2 / 32 + 1;  // words of the row mask: a bit per pair
+constexpr unsigned kAll = 0xffffffffu;
 constexpr unsigned long long kFlagAgg = 1ull << 62;
 constexpr unsigned long long kFlagInc = 2ull << 62;
 constexpr unsigned long long kValMask = (1ull << 62) - 1;
@@ -47,6 +53,24 @@ constexpr unsigned long long kWaitLimitNs = 1000000000ull;  // 1 s bound on a lo
 constexpr unsigned long long kMaxPolls = 1ull << 26;        // backstop if the timer stalls
 constexpr size_t kWsHeader = 256;                           // tile counter, padded
 constexpr int kMinTE = 64;
+
+// Staged particles: of one batch of a warp, or of one event by the CTA.
+struct Staged {
+  ffm::EvPart *part;
+  float4 *c0, *c1;  // (px, py) and (pz, E): float-float as (hi, hi, lo, lo), or two doubles
+};
+
+// One warp's part of shared memory.
+struct __align__(16) WarpBuf {
+  ffm::EvPart part[kCapW];
+  float4 c0[kCapW], c1[kCapW];
+  int4 info[32];  // by non-empty event: first particle, particles, first pair, event of the tile
+  uint32_t scale[32];  // by non-empty event: the largest high word of pt and |m|
+  int row[kCapW];      // by row: its particle, and what turns a pair's index into the partner
+  uint32_t rows[kRows];  // bit q: a row starts at pair q of the batch
+};
+static_assert(4 * sizeof(WarpBuf) >= (size_t)kCP * (sizeof(ffm::EvPart) + 2 * sizeof(float4)),
+              "an event staged by the CTA takes the place of four warps' buffers");
 
 struct JArgs {
   Lv p;
@@ -77,18 +101,9 @@ __device__ __forceinline__ void st_relaxed(unsigned long long *p, unsigned long 
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-// A float-float value kept in a double-sized shared-memory slot (its two floats' bits).
-__device__ __forceinline__ void st_ff(double *slot, const ffm::ff &x) {
-  *reinterpret_cast<float2 *>(slot) = make_float2(x.hi, x.lo);
-}
-__device__ __forceinline__ ffm::ff ld_ff(const double *slot) {
-  const float2 v = *reinterpret_cast<const float2 *>(slot);
-  return {v.x, v.y};
-}
-
 template <int NT, int LP, int LS>
-__device__ void big_event(const JArgs &A, int64_t e, int64_t pbeg, int64_t n, int64_t out0,
-                          double *s_red) {
+__device__ __noinline__ void big_event(const JArgs &A, int64_t e, int64_t pbeg, int64_t n, int64_t out0) {
+  __shared__ double s_red[4 * (NT / 32)];
   // event sum
   double acc[4] = {0, 0, 0, 0};
   for (int64_t k = threadIdx.x; k < n; k += NT) {
@@ -132,21 +147,348 @@ __device__ void big_event(const JArgs &A, int64_t e, int64_t pbeg, int64_t n, in
   if (__syncthreads_or(over) && threadIdx.x == 0) raise_status(A.status, GVX_ERR_CAPACITY);
 }
 
+// The Cartesian components of one particle in FP64, out of line (rare).
+__device__ __noinline__ void cartesian_f64(V4<double> x, double2 *xy, double2 *ze) {
+  double sn, cs;
+  sincos(x.z, &sn, &cs);
+  *xy = make_double2(x.x * cs, x.x * sn);
+  *ze = make_double2(x.x * sinh(x.y), make_leg(x).E);
+}
+
+// One particle's terms at its event's scale word wmax, to place c.  False outside the float-float
+// domain: then its scale is 0 and, with F64, its FP64 Cartesian components are staged.
+template <bool F64>
+__device__ __forceinline__ bool stage_particle(const Staged &S, int c, const V4<double> &x,
+                                               uint32_t wmax, const ffm::LcTab &T) {
+  const double pt = x.x, eta = x.y, phi = x.z, m = x.w;
+  const uint32_t hp = ffm::dhi(pt), hm = ffm::dhi(m) & 0x7fffffffu;
+  if (ffm::lc_in_domain(hp, hm, ffm::dhi(eta) & 0x7fffffffu, ffm::dhi(phi) & 0x7fffffffu, wmax)) {
+    const uint32_t ew = wmax & 0x7ff00000u, rb = ew - (127u << 20);
+    const ffm::ff ptf = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(pt), rb));
+    const ffm::ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(m), rb));
+    const int64_t ae = ffm::angle_fx(eta), ap = ffm::angle_fx(phi);
+    uint32_t n, j;
+    const ffm::ff re = ffm::fx_half_reduce(2 * ae, &n), rp = ffm::fx_half_reduce(2 * ap, &j);
+    ffm::ff sh, sn, cs;
+    const ffm::LcLeg<ffm::ff> L = ffm::lc_leg_at(ptf, mmf, re, &n, T.hyp, &sh);
+    S.part[c] = ffm::EvPart{make_float4(L.D.hi, L.Y.hi, L.D.lo, L.Y.lo), ae, ap, ptf.hi, ptf.lo, ew, 0u};
+    ffm::sincos_lc_at(rp, j, T.sin, &sn, &cs);
+    const float sphi = (ffm::dhi(phi) >> 31) ? -1.0f : 1.0f, seta = (ffm::dhi(eta) >> 31) ? -1.0f : 1.0f;
+    const ffm::ff px = ffm::lc_mul(ptf, cs), py = ffm::lc_scale(ffm::lc_mul(ptf, sn), sphi);
+    const ffm::ff pz = ffm::lc_scale(ffm::lc_mul(ptf, sh), seta);
+    S.c0[c] = make_float4(px.hi, py.hi, px.lo, py.lo);
+    S.c1[c] = make_float4(pz.hi, L.E.hi, pz.lo, L.E.lo);
+    return true;
+  }
+  if constexpr (F64) cartesian_f64(x, reinterpret_cast<double2 *>(S.c0 + c), reinterpret_cast<double2 *>(S.c1 + c));
+  S.part[c].scale = 0u;
+  return false;
+}
+
+// Two components of the sum over places c, c + step, .. < end: float-float terms of the fast-path
+// particles in *f (lanes); with F64 also the FP64 terms of the others in d, and the result is the
+// event's scale field if any particle is on the fast path (otherwise that of the last particle).
+template <bool F64>
+__device__ __forceinline__ uint32_t sum_places(const float4 *col, const ffm::EvPart *part, int c, int end,
+                                               int step, ffm::ff2 *f, double *d) {
+  ffm::ff2 a = {ffm::bc2(0.0f), ffm::bc2(0.0f)};
+  uint32_t ew = 0;
+  d[0] = d[1] = 0.0;
+  for (; c < end; c += step) {
+    const float4 v = col[c];
+    const uint32_t w = F64 ? part[c].scale : 1u;
+    if (w) {
+      a = ffm::add_same(a, ffm::ff2{ffm::mk2(v.x, v.y), ffm::mk2(v.z, v.w)});
+      ew = w;
+    } else {
+      const double2 r = *reinterpret_cast<const double2 *>(col + c);
+      d[0] += r.x;
+      d[1] += r.y;
+    }
+  }
+  if constexpr (!F64) ew = part[end - 1].scale;
+  *f = a;
+  return ew;
+}
+
+// Components 2 h and 2 h + 1 of event e's sum.
+template <int LS>
+__device__ __forceinline__ void put_sums(const JArgs &A, int64_t e, int h, double x, double y) {
+  if constexpr (LS == GVX_SOA) {
+    st_s((double *)(h ? A.sums.c[2] : A.sums.c[0]) + e, x);
+    st_s((double *)(h ? A.sums.c[3] : A.sums.c[1]) + e, y);
+  } else {
+    __stcs((double2 *)A.sums.c[0] + 2 * e + h, make_double2(x, y));
+  }
+}
+
+__device__ __forceinline__ double sum_to_double(const ffm::ff &f, uint32_t ew, double d) {
+  return ew ? ffm::lc_to_double(f, ew - (127u << 20)) + d : d;
+}
+
+// One batch by one warp: `take` events of the tile from event sb on (lane l < take having event
+// sb + l with particles lo .. hi - 1), together at most kCapW particles.  RARE: a second walk, which
+// writes the pairs that the first one left and nothing else.  Returns kOver when a pair did not
+// fit the output, kRare when a pair or an event's sums were left.
+constexpr int kOver = 1, kRare = 2;
+
+template <int LP, int LS, bool RARE>
+__device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, WarpBuf &W, int64_t e0,
+                                          int sb, int take, int64_t lo, int64_t hi, const int64_t *s_pp,
+                                          int64_t base) {
+  const int lane = threadIdx.x & 31;
+  const unsigned upto = 0xffffffffu >> (31 - lane), below = upto >> 1;
+  const Staged S = {W.part, W.c0, W.c1};
+  const int64_t pb = __shfl_sync(kAll, lo, 0);
+  const int np = (int)(__shfl_sync(kAll, hi, take - 1) - pb);
+  const int64_t q0 = s_pp[sb];
+  const int total = (int)(s_pp[sb + take] - q0);
+  // the particles' loads go out first
+  V4<double> x[2];
+#pragma unroll
+  for (int r = 0; r < 2; r++)
+    if (lane + 32 * r < np && GVX_IN_BOUNDS(pb + lane + 32 * r, A.n_particles, A.status))
+      x[r] = ld4<double, LP>(A.p, pb + lane + 32 * r);
+  // non-empty events in order; the particles they start at as bits
+  const int n_l = lane < take ? (int)(hi - lo) : 0, st_l = (int)(lo - pb);
+  const unsigned nz = __ballot_sync(kAll, n_l > 0);
+  const int nev = __popc(nz);
+  const unsigned m0 = __reduce_or_sync(kAll, n_l > 0 && st_l < 32 ? 1u << st_l : 0u);
+  const unsigned m1 = __reduce_or_sync(kAll, n_l > 0 && st_l >= 32 ? 1u << (st_l - 32) : 0u);
+  if (n_l > 0) {
+    const int k = __popc(nz & below);
+    W.info[k] = make_int4(st_l, n_l, (int)(s_pp[sb + lane] - q0), sb + lane);
+    W.scale[k] = 0u;
+  } else if (!RARE && lane < take) {
+    put_sums<LS>(A, e0 + sb + lane, 0, 0.0, 0.0);
+    put_sums<LS>(A, e0 + sb + lane, 1, 0.0, 0.0);
+  }
+  for (int w = lane; w < kRows; w += 32) W.rows[w] = 0u;
+  __syncwarp();
+  int rank[2];
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    rank[r] = r ? __popc(m0) + __popc(m1 & upto) - 1 : __popc(m0 & upto) - 1;
+    if (lane + 32 * r < np)
+      atomicMax(&W.scale[rank[r]], ffm::umax32(ffm::dhi(x[r].x), ffm::dhi(x[r].w) & 0x7fffffffu));
+  }
+  __syncwarp();
+  bool extreme = false;
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const int c = lane + 32 * r;
+    if (c < np) {
+      const int4 v = W.info[rank[r]];
+      const int li = c - v.x;
+      if (li + 1 < v.y) {  // a row: pairs first .. first + (n - li - 2), partners c + 1 ..
+        const int first = v.z + li * v.y - (li * (li + 1) >> 1);
+        W.row[c - rank[r]] = c | (c + 1 - first) << 8;
+        atomicOr(&W.rows[first >> 5], 1u << (first & 31));
+      }
+      extreme |= !stage_particle<RARE>(S, c, x[r], W.scale[rank[r]], T);
+    }
+  }
+  extreme = __any_sync(kAll, extreme);  // and the staged places are visible to the warp
+  // event sums: lanes (event, component pair, every other particle); an event with a particle
+  // outside the float-float domain gets its sums in the second walk
+  if (!RARE || extreme) {
+    for (int t = lane; t < 4 * nev; t += 32) {
+      const int4 v = W.info[t >> 2];
+      const int h = (t >> 1) & 1;
+      ffm::ff2 f;
+      double d[2];
+      uint32_t ew = sum_places<RARE>(h ? S.c1 : S.c0, S.part, v.x + (t & 1), v.x + v.y, 2, &f, d);
+      const unsigned pair = 3u << (lane & 30);
+      const ffm::ff2 g = {ffm::mk2(__shfl_xor_sync(pair, f.hi.x, 1), __shfl_xor_sync(pair, f.hi.y, 1)),
+                          ffm::mk2(__shfl_xor_sync(pair, f.lo.x, 1), __shfl_xor_sync(pair, f.lo.y, 1))};
+      if constexpr (RARE) {
+        ew |= __shfl_xor_sync(pair, ew, 1);
+        d[0] += __shfl_xor_sync(pair, d[0], 1);
+        d[1] += __shfl_xor_sync(pair, d[1], 1);
+      }
+      if ((t & 1) == 0) {
+        f = ffm::add_same(f, g);
+        put_sums<LS>(A, e0 + v.w, h, sum_to_double(ffm::lane_x(f), ew, d[0]), sum_to_double(ffm::lane_y(f), ew, d[1]));
+      }
+    }
+  }
+  // pairs
+  const int64_t dst0 = base + q0, room = A.cap - dst0;
+  const int lim = room < total ? (int)(room < 0 ? 0 : room) : total;
+  double *const out = A.pair_m + dst0;
+  bool rare = false;
+  int rows = -1;  // rows that start before the current word, less one
+  for (int r0 = 0; r0 < lim; r0 += 32) {
+    const unsigned w = W.rows[r0 >> 5];
+    const int q = r0 + lane;
+    if (q < lim) {
+      const int rec = W.row[rows + __popc(w & upto)];
+      const int i = rec & 0xff, j = q + (rec >> 8);
+      if (GVX_IN_BOUNDS(i, np, A.status) && GVX_IN_BOUNDS(j, np, A.status)) {
+        const ffm::EvPart &a = W.part[i], &b = W.part[j];
+        ffm::ff m2s;
+        const bool ok = !(extreme && (a.scale == 0u || b.scale == 0u)) && ffm::ev_pair_m2(a, b, T, &m2s);
+        if constexpr (RARE) {
+          if (!ok) st_s(out + q, pair_mass_at<LP>(A.p.c[0], A.p.c[1], A.p.c[2], A.p.c[3], pb + i, pb + j));
+        } else {
+          if (ok)
+            st_s(out + q, ffm::lc_mass_out(m2s, a.scale));
+          else
+            rare = true;
+        }
+      }
+    }
+    rows += __popc(w);
+  }
+  __syncwarp();  // before the next batch overwrites the staged particles
+  return (lim < total ? kOver : 0) | (rare || extreme ? kRare : 0);
+}
+
+// The tile's batches, every warp walking the tile and taking its turn; *large: an event was left
+// to the CTA.
+template <int NT, int LP, int LS, bool RARE>
+__device__ __forceinline__ int walk_tile(const JArgs &A, const ffm::LcTab &T, WarpBuf &W, int64_t e0,
+                                         int ne, const int64_t *s_off, const int64_t *s_pp, int64_t base,
+                                         bool *large) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int seen = 0;
+  for (int sb = 0, turn = 0; sb < ne;) {
+    const int64_t lo = s_off[min(sb + lane, ne)], hi = s_off[min(sb + lane + 1, ne)];
+    const int64_t pb = __shfl_sync(kAll, lo, 0);
+    const int take = __popc(__ballot_sync(kAll, sb + lane < ne && hi - pb <= kCapW));
+    if (take == 0) {
+      *large = true;
+      sb++;
+      continue;
+    }
+    if (turn == warp) seen |= warp_batch<LP, LS, RARE>(A, T, W, e0, sb, take, lo, hi, s_pp, base);
+    turn = turn + 1 == NT / 32 ? 0 : turn + 1;
+    sb += take;
+  }
+  return seen;
+}
+
+// One event of more than kCapW and at most kCP particles, staged by the whole CTA.
+template <int NT, int LP, int LS>
+__device__ __forceinline__ bool staged_event(const JArgs &A, const ffm::LcTab &T, const Staged &S, int64_t e,
+                                             int64_t pb, int n, int64_t out0) {
+  __shared__ uint32_t s_scale;
+  if (threadIdx.x == 0) s_scale = 0u;
+  __syncthreads();
+  for (int c = threadIdx.x; c < n; c += NT) {
+    if (!GVX_IN_BOUNDS(pb + c, A.n_particles, A.status)) continue;
+    const V4<double> x = ld4c<LP>(A.p, pb + c);
+    atomicMax(&s_scale, ffm::umax32(ffm::dhi(x.x), ffm::dhi(x.w) & 0x7fffffffu));
+  }
+  __syncthreads();
+  for (int c = threadIdx.x; c < n; c += NT) {
+    if (!GVX_IN_BOUNDS(pb + c, A.n_particles, A.status)) continue;
+    stage_particle<true>(S, c, ld4c<LP>(A.p, pb + c), s_scale, T);
+  }
+  __syncthreads();
+  if (threadIdx.x < 2) {
+    ffm::ff2 f;
+    double d[2];
+    const uint32_t ew = sum_places<true>(threadIdx.x ? S.c1 : S.c0, S.part, 0, n, 1, &f, d);
+    put_sums<LS>(A, e, threadIdx.x, sum_to_double(ffm::lane_x(f), ew, d[0]), sum_to_double(ffm::lane_y(f), ew, d[1]));
+  }
+  const int total = n * (n - 1) / 2;
+  bool fits = true;
+  for (int q = threadIdx.x; q < total; q += NT) {
+    int i, j;
+    decode_pair32(q, n, i, j);
+    if (!(GVX_IN_BOUNDS(i, n, A.status) && GVX_IN_BOUNDS(j, n, A.status))) continue;
+    if (out0 + q >= A.cap) {
+      fits = false;
+      continue;
+    }
+    const ffm::EvPart &a = S.part[i], &b = S.part[j];
+    ffm::ff m2s;
+    if (a.scale != 0u && b.scale != 0u && ffm::ev_pair_m2(a, b, T, &m2s))
+      st_s(A.pair_m + out0 + q, ffm::lc_mass_out(m2s, a.scale));
+    else
+      st_s(A.pair_m + out0 + q, pair_mass_at<LP>(A.p.c[0], A.p.c[1], A.p.c[2], A.p.c[3], pb + i, pb + j));
+  }
+  __syncthreads();
+  return fits;
+}
+
+// What the batches of a tile left, by the whole CTA.
+template <int NT, int LP, int LS>
+__device__ __noinline__ void finish_tile(const JArgs &A, unsigned char *s_dyn, int64_t e0, int ne,
+                                         const int64_t *s_off, const int64_t *s_pp, int64_t base, bool rare) {
+  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
+  bool large;
+  if (rare)
+    walk_tile<NT, LP, LS, true>(A, T, reinterpret_cast<WarpBuf *>(s_dyn)[threadIdx.x >> 5], e0, ne, s_off, s_pp,
+                                base, &large);
+  __syncthreads();
+  Staged S;
+  S.part = reinterpret_cast<ffm::EvPart *>(s_dyn);
+  S.c0 = reinterpret_cast<float4 *>(S.part + kCP);
+  S.c1 = S.c0 + kCP;
+  for (int e = 0; e < ne; e++) {
+    const int64_t pb = s_off[e], n = s_off[e + 1] - pb;
+    if (n <= kCapW) continue;
+    bool fits = true;
+    if (n <= kCP)
+      fits = staged_event<NT, LP, LS>(A, T, S, e0 + e, pb, (int)n, base + s_pp[e]);
+    else
+      big_event<NT, LP, LS>(A, e0 + e, pb, n, base + s_pp[e]);
+    if (!fits) raise_status(A.status, GVX_ERR_CAPACITY);
+  }
+  __syncthreads();
+}
+
+// The pairs before tile `tile`, by one warp: its own total published first, then the descriptors
+// before it read 32 at a time, back to the nearest inclusive prefix.
+__device__ __forceinline__ int64_t look_back(const JArgs &A, int64_t tile, int64_t tile_total) {
+  const int lane = threadIdx.x & 31;
+  int64_t prefix = 0;
+  if (tile > 0) {
+    if (lane == 0) st_relaxed(&A.desc[tile], kFlagAgg | (unsigned long long)tile_total);
+    unsigned long long t0 = 0, polls = 0;
+    for (int64_t j = tile - 1; j >= 0;) {
+      // lane l: descriptor j - l; before the first tile there is an inclusive prefix of 0
+      const unsigned long long d = j - lane >= 0 ? ld_relaxed(&A.desc[j - lane]) : kFlagInc;
+      const unsigned long long f = d & ~kValMask;
+      const unsigned inc = __ballot_sync(kAll, f == kFlagInc), none = __ballot_sync(kAll, f == 0);
+      const int last = inc ? __ffs((int)inc) - 1 : 31;  // the words up to `last` are needed
+      if (none & (0xffffffffu >> (31 - last))) {
+        const unsigned long long now = global_ns();
+        if (t0 == 0) t0 = now;
+        const bool give_up = now - t0 > kWaitLimitNs || ++polls > kMaxPolls;
+        if (__any_sync(kAll, give_up)) {
+          if (lane == 0) raise_status(A.status, GVX_ERR_TIMEOUT);
+          break;
+        }
+        __nanosleep(64);
+        continue;
+      }
+      int64_t v = lane <= last ? (int64_t)(d & kValMask) : 0;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kAll, v, o);
+      prefix += v;
+      if (inc) break;
+      j -= 32;
+    }
+  }
+  if (lane == 0) st_relaxed(&A.desc[tile], kFlagInc | (unsigned long long)(prefix + tile_total));
+  return prefix;
+}
+
 template <int TE, int NT, int LP, int LS>
-__global__ void __launch_bounds__(NT, 1024 / NT) event_pairs_kernel(JArgs A) {
-  static_assert(TE <= NT && NT % 32 == 0, "one event per thread in the tile scan");
-  extern __shared__ double s_dyn[];
-  double *s_eta = s_dyn, *s_phi = s_eta + kCP, *s_px = s_phi + kCP, *s_py = s_px + kCP;
-  double *s_pz = s_py + kCP, *s_E = s_pz + kCP;
-  ffm::ff *s_pt = reinterpret_cast<ffm::ff *>(s_E + kCP), *s_Y = s_pt + kCP, *s_D = s_Y + kCP;
-  int *s_sc = reinterpret_cast<int *>(s_D + kCP), *s_fs = s_sc + kCP;
+__global__ void __launch_bounds__(NT, 768 / NT) event_pairs_kernel(const __grid_constant__ JArgs A) {
+  static_assert(TE <= NT && NT % 128 == 0, "one event per thread in the tile scan");
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  WarpBuf *bufs = reinterpret_cast<WarpBuf *>(s_dyn);
   __shared__ int64_t s_off[TE + 1];
   __shared__ int64_t s_pp[TE + 1];
   __shared__ int64_t s_warp[NT / 32];
-  __shared__ double s_red[4 * (NT / 32)];
   __shared__ int64_t s_base;
   __shared__ int64_t s_tile;
   const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   for (;;) {
     if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(A.counter, 1u);
@@ -182,181 +524,21 @@ __global__ void __launch_bounds__(NT, 1024 / NT) event_pairs_kernel(JArgs A) {
     if (threadIdx.x == 0) s_pp[ne] = tile_total;
 
     // 2. decoupled look-back
-    if (threadIdx.x == 0) {
-      int64_t prefix = 0;
-      if (tile == 0) {
-        st_relaxed(&A.desc[0], kFlagInc | (unsigned long long)tile_total);
-      } else {
-        st_relaxed(&A.desc[tile], kFlagAgg | (unsigned long long)tile_total);
-        int64_t j = tile - 1;
-        unsigned long long t0 = 0, polls = 0;
-        while (j >= 0) {
-          unsigned long long d = ld_relaxed(&A.desc[j]);
-          unsigned long long f = d & ~kValMask;
-          if (f == 0) {
-            unsigned long long now = global_ns();
-            if (t0 == 0) t0 = now;
-            if (now - t0 > kWaitLimitNs || ++polls > kMaxPolls) {
-              raise_status(A.status, GVX_ERR_TIMEOUT);
-              break;
-            }
-            __nanosleep(64);
-            continue;
-          }
-          prefix += (int64_t)(d & kValMask);
-          if (f == kFlagInc) break;
-          j--;
-        }
-        st_relaxed(&A.desc[tile], kFlagInc | (unsigned long long)(prefix + tile_total));
-      }
-      s_base = prefix;
+    if (warp == 0) {
+      const int64_t prefix = look_back(A, tile, tile_total);
+      if (lane == 0) s_base = prefix;
     }
     __syncthreads();
     const int64_t base = s_base;
     if (threadIdx.x < ne) A.pair_off[e0 + threadIdx.x] = base + s_pp[threadIdx.x];
     if (tile == A.n_tiles - 1 && threadIdx.x == 0) A.pair_off[A.n_events] = base + tile_total;
 
-    // 3./4. sub-batches of whole events that fit in shared memory
-    int sb = 0;
-    while (sb < ne) {
-      const int64_t pb = s_off[sb];
-      const bool fits = threadIdx.x >= sb && threadIdx.x < ne && s_off[threadIdx.x + 1] - pb <= kCP;
-      const int sbe = sb + __syncthreads_count(fits);
-      if (sbe == sb) {  // one event larger than the staging buffer
-        const int64_t n = s_off[sb + 1] - pb;
-        big_event<NT, LP, LS>(A, e0 + sb, pb, n, base + s_pp[sb], s_red);
-        sb++;
-        __syncthreads();
-        continue;
-      }
-      const int np = (int)(s_off[sbe] - pb);
-      // (a) raw particles; pt and m parked in the px/py slots, the larger high word of pt and
-      // |m| in s_sc
-      for (int k = threadIdx.x; k < np; k += NT) {
-        if (!GVX_IN_BOUNDS(pb + k, A.n_particles, A.status)) continue;
-        V4<double> v = ld4<double, LP>(A.p, pb + k);
-        s_eta[k] = v.y;
-        s_phi[k] = v.z;
-        s_px[k] = v.x;
-        s_py[k] = v.w;
-        s_sc[k] = (int)ffm::umax32(ffm::dhi(v.x), ffm::dhi(v.w) & 0x7fffffffu);
-      }
-      __syncthreads();
-      // (b) one thread per particle: its event's scale (the largest high word over the event,
-      // from s_sc), whether the fast path takes it (the event's scale field goes to s_fs, so s_sc
-      // stays intact for the other particles of the event), and its per-particle terms
-      for (int k = threadIdx.x; k < np; k += NT) {
-        int lo = sb, hi = sbe - 1;  // the particle's event: the last e with s_off[e] <= pb + k
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (s_off[mid] <= pb + k) lo = mid;
-          else hi = mid - 1;
-        }
-        uint32_t wmax = 0;
-        for (int t = (int)(s_off[lo] - pb); t < (int)(s_off[lo + 1] - pb); t++)
-          wmax = ffm::umax32((uint32_t)s_sc[t], wmax);
-        const double pt = s_px[k], eta = s_eta[k], phi = s_phi[k], m = s_py[k];
-        // the domain of the elementwise fast path (mass_lc.cuh), at the event's scale
-        const uint32_t ew = wmax & 0x7ff00000u;
-        const uint32_t hp = ffm::dhi(pt), hm = ffm::dhi(m) & 0x7fffffffu;
-        const uint32_t he = ffm::dhi(eta) & 0x7fffffffu, hf = ffm::dhi(phi) & 0x7fffffffu;
-        int sc = wmax - (200u << 20) < (1700u << 20) &&
-                         ffm::umin32(hp - 0x100000u, hm - 0x100000u) >= ew - (41u << 20) &&
-                         ffm::umax32(hp, hm) >= 0x100000u && he < 0x40200000u && hf < 0x400C0000u
-                     ? (int)ew
-                     : kNoFast;
-        if (sc != kNoFast) {
-          const uint32_t rb = ew - (127u << 20);
-          const ffm::ff ptf = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(pt), rb));
-          const ffm::ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(m), rb));
-          const ffm::ff xe = ffm::cvt1(ffm::cvt_parts_normal(ffm::umax32(he, 0x3E100000u),
-                                                             ffm::dlo(eta), ffm::kRebaseOne));
-          ffm::ff sh, sn, cs;
-          const ffm::LcLeg<ffm::ff> L = ffm::lc_leg(ptf, mmf, xe, T.hyp, &sh);
-          ffm::sincos_lc(ffm::cvt1(ffm::cvt_parts(hf, ffm::dlo(phi), ffm::kRebaseOne)), T.sin, &sn, &cs);
-          s_pt[k] = ptf;
-          s_Y[k] = L.Y;
-          s_D[k] = L.D;
-          // the Cartesian components in float-float at the event's scale (summed per event in
-          // float-float and converted once per event: no FP64 operation per particle)
-          const float sphi = (ffm::dhi(phi) >> 31) ? -1.0f : 1.0f, seta = (ffm::dhi(eta) >> 31) ? -1.0f : 1.0f;
-          st_ff(s_px + k, ffm::lc_mul(ptf, cs));
-          st_ff(s_py + k, ffm::lc_scale(ffm::lc_mul(ptf, sn), sphi));
-          st_ff(s_pz + k, ffm::lc_scale(ffm::lc_mul(ptf, sh), seta));
-          st_ff(s_E + k, L.E);
-        } else {  // FP64 evaluation
-          double sphi, cphi;
-          sincos(phi, &sphi, &cphi);
-          s_px[k] = pt * cphi;
-          s_py[k] = pt * sphi;
-          s_pz[k] = pt * sinh(eta);
-          s_E[k] = make_leg(V4<double>{pt, eta, phi, m}).E;
-        }
-        s_fs[k] = sc;
-      }
-      __syncthreads();
-      // event sums: one thread per (event, component), taken by the last threads of the CTA (those
-      // with one pair fewer in the pair loop's last round); float-float terms of the fast-path
-      // particles summed in float-float at the event's scale, FP64 terms of the others in FP64
-      for (int t = NT - 1 - (int)threadIdx.x; t < 4 * (sbe - sb); t += NT) {
-        const int e = sb + (t >> 2), c = t & 3;
-        const double *col = c == 0 ? s_px : c == 1 ? s_py : c == 2 ? s_pz : s_E;
-        ffm::ff sf = {0.0f, 0.0f};
-        double sd = 0.0;
-        int sce = kNoFast;
-        const int k1 = (int)(s_off[e + 1] - pb);
-        for (int k = (int)(s_off[e] - pb); k < k1; k++) {
-          if (s_fs[k] != kNoFast) {
-            sf = ffm::add_same(sf, ld_ff(col + k));
-            sce = s_fs[k];
-          } else {
-            sd += col[k];
-          }
-        }
-        const double total = sce != kNoFast ? ffm::lc_to_double(sf, (uint32_t)sce - (127u << 20)) + sd : sd;
-        double *dst = LS == GVX_SOA ? (double *)A.sums.c[c] + (e0 + e) : (double *)A.sums.c[0] + 4 * (e0 + e) + c;
-        st_s(dst, total);
-      }
-      const int64_t q0 = s_pp[sb], q1 = s_pp[sbe];
-      bool over = false;
-      for (int64_t q = q0 + threadIdx.x; q < q1; q += NT) {
-        int lo = sb, hi = sbe - 1;
-        while (lo < hi) {
-          int mid = (lo + hi + 1) >> 1;
-          if (s_pp[mid] <= q) lo = mid;
-          else hi = mid - 1;
-        }
-        const int64_t n = s_off[lo + 1] - s_off[lo];
-        int64_t i, j;
-        decode_pair(q - s_pp[lo], n, i, j);
-        const int ia = (int)(s_off[lo] - pb + i), ib = (int)(s_off[lo] - pb + j);
-        if (!(GVX_IN_BOUNDS(ia, np, A.status) && GVX_IN_BOUNDS(ib, np, A.status))) continue;
-        double mass;
-        bool done = false;
-        const int sc = s_fs[ia];
-        if (sc != kNoFast && s_fs[ib] != kNoFast) {
-          ffm::ff S, m2s;
-          const bool oks = ffm::lc_pair_S(s_eta[ia], s_eta[ib], s_phi[ia], s_phi[ib], T, &S);
-          if (ffm::lc_pair_m2(s_pt[ia], s_pt[ib], s_Y[ia], s_Y[ib], s_D[ia], s_D[ib], S, &m2s) && oks) {
-            mass = ffm::lc_mass_out_int(m2s, (uint32_t)sc);
-            done = true;
-          }
-        }
-        if (!done) {
-          Leg<double> a = make_leg(ld4<double, LP>(A.p, pb + ia));
-          Leg<double> b = make_leg(ld4<double, LP>(A.p, pb + ib));
-          mass = sqrt(pair_terms(a, b).m2);
-        }
-        const int64_t dst = base + q;
-        if (dst < A.cap)
-          st_s(A.pair_m + dst, mass);
-        else
-          over = true;
-      }
-      if (__syncthreads_or(over) && threadIdx.x == 0) raise_status(A.status, GVX_ERR_CAPACITY);
-      sb = sbe;
-    }
-    __syncthreads();
+    // 3. the batches, 4. what they leave
+    bool large = false;
+    const int seen = walk_tile<NT, LP, LS, false>(A, T, bufs[warp], e0, ne, s_off, s_pp, base, &large);
+    if ((seen & kOver) && lane == 0) raise_status(A.status, GVX_ERR_CAPACITY);
+    const bool rare = __syncthreads_or(seen & kRare);
+    if (rare || large) finish_tile<NT, LP, LS>(A, s_dyn, e0, ne, s_off, s_pp, base, rare);
   }
 }
 
@@ -370,6 +552,7 @@ constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
 template <int TE, int NT, int LP, int LS>
 cudaError_t launch_shape(const JArgs &A0, bool skip_first_tile, cudaStream_t s) {
   auto kern = event_pairs_kernel<TE, NT, LP, LS>;
+  constexpr size_t kDynSmem = (NT / 32) * sizeof(WarpBuf);
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kDynSmem);
   if (err != cudaSuccess) return err;
