@@ -2,9 +2,9 @@
 // are templated on their coordinate system; Sec. 4.1: transformations are 4x4 matrices applied
 // to every vector of an array).
 //
-// gvx_invariant_mass_cart: pair masses of Cartesian legs, PxPyPzE or PxPyPzM, through the
-// fixed-point evaluations of cart_fixed.cuh (integer and FP32 pipes); the rare pairs outside
-// their domain take the cancellation-free FP64 form of cart_mass.cuh (an FMA-exact cross product
+// gvx_invariant_mass_cart: pair masses of Cartesian legs, PxPyPzE through the fixed-point evaluation
+// of cart_fixed.cuh (integer and FP32 pipes), PxPyPzM through the float-float one of
+// cart_pxpypzm.cuh; the rare pairs outside their domain take the cancellation-free FP64 form of cart_mass.cuh (an FMA-exact cross product
 // and E^2 - |p|^2), on the FP64 pipe for both storage precisions.
 //
 // gvx_to_pxpypze: PtEtaPhiM, PtEtaPhiE or PxPyPzM vectors to PxPyPzE (convert_ff.cuh in FP64 with

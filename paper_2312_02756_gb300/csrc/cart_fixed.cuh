@@ -189,140 +189,7 @@ GVX_HD bool mass_pxpypze(const float *a, const float *b, float *out) {
   return true;
 }
 
-// ---- PxPyPzM legs ----------------------------------------------------------------------------
-// With the mass stored, E_i = sqrt(P_i^2 + m_i^2) is not a stored number, and
-//   m^2 = m1^2 + m2^2 + 2 (E1 E2 - p1.p2),
-//   E1 E2 - p1.p2 = (|p1 x p2|^2 + m1^2 P2^2 + m2^2 P1^2 + m1^2 m2^2) / (E1 E2 + p1.p2)   (p1.p2 > 0)
-//                 = E1 E2 + |p1.p2|                                                        (otherwise),
-// the numerator being E1^2 E2^2 - (p1.p2)^2 by Lagrange's identity.  Every term is non-negative
-// and the only cancelling quantities are the components of p1 x p2: those come from the
-// fixed-point limb products (components truncated to units of 2^-83 of their leg's scale, the
-// products kept to units of 2^-102 of 2^(s1 + s2)); P_i^2, m_i^2 and p1.p2 (which only ever
-// enters next to E1 E2) are float-float arithmetic on the scaled components, like the rest.
-// Each leg has its own power-of-two scale 2^s_i: an absolute error in m_i^2 reaches m^2
-// multiplied by about E_o / E_i, so the resolution must follow each leg.  In units of the larger
-// leg's squared scale H the fixed-point errors stay below 2^-76; the result is kept when
-// m^2 >= 2^-31 H, so its relative error (with the float-float steps) is below 2^-43.
-// Domain: both legs finite with scale exponents within half the format's limit and at most 60
-// apart.
-
-// (A B) / 2^64 for magnitudes A, B < 2^85, within 4 units: with A = ah 2^64 + a1 2^32 + a0,
-// A B / 2^64 = ah bh 2^64 + ah (b1 2^32 + b0) + bh (a1 2^32 + a0) + a1 b1 + (a1 b0 + a0 b1) / 2^32
-// + a0 b0 / 2^64, the last term dropped and the one before it truncated term by term.
-GVX_HD u128 mul_shift64(u128 A, u128 B) {
-  const uint32_t ah = (uint32_t)(A >> 64), a1 = (uint32_t)((uint64_t)A >> 32), a0 = (uint32_t)A;
-  const uint32_t bh = (uint32_t)(B >> 64), b1 = (uint32_t)((uint64_t)B >> 32), b0 = (uint32_t)B;
-  return ((u128)((uint64_t)ah * bh) << 64) + mul32x64(ah, (uint64_t)B) + mul32x64(bh, (uint64_t)A) +
-         ((uint64_t)a1 * b1 + mul32hi(a1, b0) + mul32hi(a0, b1));
-}
-
-// |q| * 2^-102 as ff (truncated to 47 bits), for any q < 2^112; 0 gives 0.
-GVX_HD ff fixed_to_ff_any(u128 q) {
-  const uint64_t hi64 = (uint64_t)(q >> 64), lo64 = (uint64_t)q;
-  if ((hi64 | lo64) == 0) return {0.0f, 0.0f};
-#if defined(__CUDA_ARCH__)
-  const int p = hi64 ? 127 - __clzll((long long)hi64) : 63 - __clzll((long long)lo64);
-#else
-  const int p = hi64 ? 127 - __builtin_clzll(hi64) : 63 - __builtin_clzll(lo64);
-#endif
-  const uint64_t t = p >= 46 ? (uint64_t)(q >> (p - 46)) : lo64 << (46 - p);
-  const uint32_t top = (uint32_t)(t >> 23), rest = (uint32_t)t & 0x7fffffu;
-  const uint32_t eh = (uint32_t)(p - kM2Units + 127);  // >= 25
-  const float hi = ffm::u2f((eh << 23) | (top & 0x7fffffu));
-  const uint32_t base = (eh - 23u) << 23;
-  return {hi, ffm::fsub(ffm::u2f(base | rest), ffm::u2f(base))};
-}
-
-// x 2^-s as ff: a double through the ranged conversion (below 2^-74 counts as 0), a float exactly.
-GVX_HD ff scaled_ff(double x, int s) { return ffm::from_double_ranged(x, s); }
-GVX_HD ff scaled_ff(float x, int s) { return {ffm::fmul(x, ffm::pow2f(-s)), 0.0f}; }
-
-// |component of p1 x p2| = |s_a A - s_b B| for the magnitudes A, B of the two products.
-GVX_HD ff cross_component(u128 A, bool na, u128 B, bool nb) {
-  return fixed_to_ff_any(abs_sum(A, na, B, !nb));
-}
-
-// The scaled mass sqrt(m^2 / 2^(2 e)) in ff and the exponent e of the pair mass of two PxPyPzM
-// legs; false outside the fast path.
-template <typename T>
-GVX_HD bool mass_pxpypzm_scaled(const T *a, const T *b, ff *m, int *e_out) {
-  Decoded d[8];
-  int e1 = 0, e2 = 0;
-#pragma unroll
-  for (int k = 0; k < 4; k++) {
-    d[k] = decode(a[k]);
-    d[k + 4] = decode(b[k]);
-    e1 = d[k].e > e1 ? d[k].e : e1;
-    e2 = d[k + 4].e > e2 ? d[k + 4].e : e2;
-  }
-  const int s1 = e1 - Fmt<T>::kBias, s2 = e2 - Fmt<T>::kBias;
-  const int lim = Fmt<T>::kScaleLim / 2;
-  if (e1 == Fmt<T>::kMaxE || e2 == Fmt<T>::kMaxE || s1 < -lim || s1 > lim || s2 < -lim || s2 > lim ||
-      s1 - s2 > 60 || s2 - s1 > 60)
-    return false;
-  using namespace ffm;
-  // |p1 x p2| components from exact limb products (scale 2^(s1 + s2))
-  u128 A[3], B[3];
-#pragma unroll
-  for (int k = 0; k < 3; k++) {
-    A[k] = align<T>(d[k], e1);
-    B[k] = align<T>(d[k + 4], e2);
-  }
-  const ff cx = cross_component(mul_shift64(A[1], B[2]), d[1].neg != d[6].neg,
-                                mul_shift64(A[2], B[1]), d[2].neg != d[5].neg);
-  const ff cy = cross_component(mul_shift64(A[2], B[0]), d[2].neg != d[4].neg,
-                                mul_shift64(A[0], B[2]), d[0].neg != d[6].neg);
-  const ff cz = cross_component(mul_shift64(A[0], B[1]), d[0].neg != d[5].neg,
-                                mul_shift64(A[1], B[0]), d[1].neg != d[4].neg);
-  // the rest in ff on the scaled components; the per-leg quantities |p_i|^2, m_i^2 and E_i^2
-  // of both legs on paired FP32 operations (mass_ff2.cuh: lane x leg 1, lane y leg 2, each lane
-  // the scalar operations' bits)
-  ff2 v[4];
-#pragma unroll
-  for (int k = 0; k < 4; k++) v[k] = pack(scaled_ff(a[k], s1), scaled_ff(b[k], s2));
-  const ff2 PP = add_same(add_same(sqr(v[0]), sqr(v[1])), sqr(v[2]));
-  const ff2 qq = sqr(v[3]);
-  const ff2 EE = add_same(PP, qq);
-  const ff P1 = lane_x(PP), P2 = lane_y(PP), q1 = lane_x(qq), q2 = lane_y(qq);
-  const ff dot = add(add(mul(lane_x(v[0]), lane_y(v[0])), mul(lane_x(v[1]), lane_y(v[1]))),
-                     mul(lane_x(v[2]), lane_y(v[2])));
-  const ff E1E2 = ffm::sqrt(mul(lane_x(EE), lane_y(EE)));  // scale 2^(s1 + s2)
-  ff T2;
-  if (dot.hi > 0.0f) {
-    const ff c2 = add_same(add_same(sqr(cx), sqr(cy)), sqr(cz));
-    const ff N = add_same(add_same(c2, mul(q1, P2)), add_same(mul(q2, P1), mul(q1, q2)));
-    T2 = scale(div(N, add_same(E1E2, dot)), 2.0f);
-  } else {
-    T2 = scale(add_same(E1E2, neg(dot)), 2.0f);
-  }
-  // m^2 / 2^(s1 + s2) = q1 2^(s1 - s2) + q2 2^(s2 - s1) + 2 T; an odd s1 + s2 moves one factor 2
-  // inside the root
-  const int odd = (s1 + s2) & 1;
-  const ff m2 = renorm(add_same(add_same(scale(q1, pow2f(s1 - s2 + odd)), scale(q2, pow2f(s2 - s1 + odd))),
-                                scale(T2, odd ? 2.0f : 1.0f)));
-  // threshold: m^2 >= 2^-31 2^(2 max(s1, s2)), i.e. the scaled value >= 2^(|s1 - s2| - 31 + odd)
-  const int gap = s1 > s2 ? s1 - s2 : s2 - s1;
-  if (!(m2.hi >= pow2f(gap - 31 + odd))) return false;
-  *m = ffm::sqrt(m2);
-  *e_out = (s1 + s2 - odd) / 2;
-  return true;
-}
-
-GVX_HD bool mass_pxpypzm(const double *a, const double *b, double *out) {
-  ff m;
-  int e;
-  if (!mass_pxpypzm_scaled(a, b, &m, &e)) return false;
-  *out = ffm::to_double(m, e);
-  return true;
-}
-
-GVX_HD bool mass_pxpypzm(const float *a, const float *b, float *out) {
-  ff m;
-  int e;
-  if (!mass_pxpypzm_scaled(a, b, &m, &e)) return false;
-  *out = ffm::fmul(ffm::fadd(m.hi, m.lo), ffm::pow2f(e));
-  return true;
-}
-
 }  // namespace cfix
 }  // namespace gvx
+
+#include "cart_pxpypzm.cuh"
