@@ -271,21 +271,28 @@ GVX_HD ff from_double(double d, bool *ok, int shift = 0) {
   return {u2f(hib), sign ? -lo : lo};
 }
 
+// (hi:lo << 3) >> 32: the top word of a double shifted left by three bits.
+GVX_HD uint32_t funnel_l3(uint32_t lo, uint32_t hi) {
+#if defined(__CUDA_ARCH__)
+  return __funnelshift_l(lo, hi, 3);
+#else
+  return (hi << 3) | (lo >> 29);
+#endif
+}
+
 // from_double without the range checks, for a d whose scaled magnitude is known to be below
-// 2^126: zeros, denormals and values that scale below 2^-74 give a signed zero.  Bitwise the same
-// result as from_double wherever that leaves *ok set.
+// 2^126: zeros, denormals and values that scale below 2^-74 give a signed zero.
+// Bitwise the same result as from_double wherever that leaves *ok set.  The rounding is one addition
+// below hi's last bit, whose carry runs through the fraction into the exponent.
 GVX_HD ff from_double_ranged(double d, int shift) {
-  uint32_t wh = dhi(d), wl = dlo(d);
-  uint32_t sign = wh & 0x80000000u;
-  int e = (int)((wh >> 20) & 0x7ffu);
-  int ef = e - 896 - shift;
-  uint32_t top = ((wh & 0xfffffu) << 3) | (wl >> 29);
-  uint32_t rbit = (wl >> 28) & 1u;
-  uint32_t hib = (sign | ((uint32_t)ef << 23) | top) + rbit;
-  int32_t rem = (int32_t)(wl & 0x1fffffffu) - (int32_t)(rbit << 29);
-  float lo = fmul(i2f(rem), pow2f(ef - 179));
-  ff r = {u2f(hib), sign ? -lo : lo};
-  return (e != 0 && ef >= 53) ? r : ff{u2f(sign), 0.0f};
+  const uint32_t wh = dhi(d), wl = dlo(d), sign = wh & 0x80000000u;
+  const uint32_t w = (wh & 0x7fffffffu) - ((uint32_t)(896 + shift) << 20);  // the exponent rebased
+  const uint32_t rl = wl + 0x10000000u;
+  const uint32_t hib = funnel_l3(rl, w + (rl < wl ? 1u : 0u)) | sign;
+  const int32_t rem = (int32_t)(wl << 3) >> 3;  // what hi leaves, in units of its last bit 2^-29
+  const uint32_t unit = (((w << 3) & 0x7f800000u) - (52u << 23)) | sign;
+  const bool ok = (int32_t)w >= (53 << 20) && (wh & 0x7ff00000u) != 0u;
+  return {u2f(ok ? hib : sign), u2f(ok ? f2u(fmul(i2f(rem), u2f(unit))) : 0u)};
 }
 
 // Biased exponent field of a double (0 for zero and denormals).

@@ -61,15 +61,6 @@ GVX_HD gvx_f4 ldtab(const gvx_f4 *p) {
 GVX_HD uint32_t umax32(uint32_t a, uint32_t b) { return a > b ? a : b; }
 GVX_HD uint32_t umin32(uint32_t a, uint32_t b) { return a < b ? a : b; }
 
-// (hi:lo << 3) >> 32: the top word of a double shifted left by three bits.
-GVX_HD uint32_t funnel_l3(uint32_t lo, uint32_t hi) {
-#if defined(__CUDA_ARCH__)
-  return __funnelshift_l(lo, hi, 3);
-#else
-  return (hi << 3) | (lo >> 29);
-#endif
-}
-
 // Hardware approximations (MUFU): 1/a and 1/sqrt(a) with a relative error below 2^-22.9.  The
 // host build models that worst case (the result moved by +-2^-23 relative, the sign taken from
 // the input's bits), so that the host tests bound the device's error rather than a correctly
