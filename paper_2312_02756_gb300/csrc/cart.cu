@@ -74,20 +74,36 @@ __global__ void __launch_bounds__(256, 4) lorentz_apply_kernel(const T *__restri
     __shared__ double s_raw[16];
     __shared__ int s_r[4];
     __shared__ int s_ok;
-    if (threadIdx.x < 16) s_raw[threadIdx.x] = L[threadIdx.x];
-    if (threadIdx.x == 0) {
-      double l0[16];
-      for (int k = 0; k < 16; k++) l0[k] = L[k];
-      const ffm::LorentzFF M = ffm::lorentz_ff(l0);
-      ffm::pair_rows(M, s_l);
-      for (int k = 0; k < 4; k++) s_r[k] = M.r[k];
-      s_ok = M.ok;
-    }
-    __syncthreads();
-    const bool ok = s_ok != 0;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     V4<T> xn = {0, 0, 0, 0};
     if (i < n) xn = ld4<T, LV>(v, i);
+    // lorentz_ff and pair_rows, one entry per lane of the first warp: by one thread the sixteen
+    // conversions held up each block's start (a quarter of the stalls were at the barrier; 2^24 vectors
+    // 200 us, 191 us so and with the shorter conversion of ff.cuh)
+    if (threadIdx.x < 32) {
+      const int k = threadIdx.x & 15, row = k >> 2, p = row >> 1, y = row & 1;
+      const double l = L[k];
+      const uint32_t hl = ffm::dhi(l) & 0x7fffffffu;
+      int e = ffm::dexp(l);
+      e = max(e, __shfl_xor_sync(0xffffffffu, e, 1));
+      e = max(e, __shfl_xor_sync(0xffffffffu, e, 2));
+      const unsigned nz = __ballot_sync(0xffffffffu, (hl | ffm::dlo(l)) != 0u);
+      const bool any = ((nz >> (4 * row)) & 15u) != 0u;
+      const int r = any ? e - 1023 : 0;
+      const bool ok = !any || (r >= -ffm::kApplyScaleLim && r <= ffm::kApplyScaleLim);
+      const bool all = __all_sync(0xffffffffu, ok);
+      const ffm::ff f = ffm::from_double_ranged(l, r);
+      if (threadIdx.x < 16) {
+        s_raw[k] = l;
+        float *q = reinterpret_cast<float *>(&s_l[4 * p + (k & 3)]);
+        q[y] = f.hi;
+        q[2 + y] = f.lo;
+        if ((k & 3) == 0) s_r[row] = r;
+        if (k == 0) s_ok = all;
+      }
+    }
+    __syncthreads();
+    const bool ok = s_ok != 0;
     for (; i < n; i += stride) {
       // the next vector's loads go out before this one's arithmetic: two vectors in flight
       const V4<T> x = xn;
