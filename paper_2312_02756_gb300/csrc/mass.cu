@@ -53,6 +53,34 @@ __global__ void __launch_bounds__(256) mass_kernel(Lv a, Lv b, T *__restrict__ m
   }
 }
 
+// FP32, both legs as columns on 16-byte boundaries: four consecutive pairs per thread and step, eight
+// loads and one store of 16 bytes in place of 32 and four.  2^26 pairs: 374 us (95% of the copy rate)
+// against 428 us for the kernel above, which is short of issue slots.
+__global__ void __launch_bounds__(256) mass_f32_x4_kernel(Lv a, Lv b, float *__restrict__ m, int64_t n) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, n4 = n / 4;
+  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  for (int64_t i = t; i < n4; i += stride) {
+    float4 x[4], y[4], r;
+#pragma unroll
+    for (int c = 0; c < 4; c++) {
+      x[c] = __ldcs((const float4 *)a.c[c] + i);
+      y[c] = __ldcs((const float4 *)b.c[c] + i);
+    }
+    const auto pair = [](const V4<float> &u, const V4<float> &v) {
+      return sqrt_(pair_terms(make_leg(u), make_leg(v)).m2);
+    };
+    r.x = pair({x[0].x, x[1].x, x[2].x, x[3].x}, {y[0].x, y[1].x, y[2].x, y[3].x});
+    r.y = pair({x[0].y, x[1].y, x[2].y, x[3].y}, {y[0].y, y[1].y, y[2].y, y[3].y});
+    r.z = pair({x[0].z, x[1].z, x[2].z, x[3].z}, {y[0].z, y[1].z, y[2].z, y[3].z});
+    r.w = pair({x[0].w, x[1].w, x[2].w, x[3].w}, {y[0].w, y[1].w, y[2].w, y[3].w});
+    __stcs((float4 *)m + i, r);
+  }
+  if (t < n - 4 * n4) {
+    const int64_t i = 4 * n4 + t;
+    st_s(m + i, sqrt_(pair_terms(make_leg(ld4<float, GVX_SOA>(a, i)), make_leg(ld4<float, GVX_SOA>(b, i))).m2));
+  }
+}
+
 // FP64 forward: grid-stride, one pair per thread and step; 64 registers, eight CTAs of 128
 // threads per SM, a grid of 32 times the resident CTAs (small CTAs and many waves even out the
 // SMs' progress: 2-3% faster than four CTAs of 256 and 8 waves on GB300).  For a leg in SoA layout (four separate arrays), lanes 0..7 of each warp
@@ -209,7 +237,12 @@ template <typename T>
 cudaError_t launch_mass_t(const Lv &a, const Lv &b, void *m, int64_t n, cudaStream_t s) {
   const int threads = 256;
   T *mo = (T *)m;
-  if (a.layout == GVX_SOA && b.layout == GVX_SOA)
+  uintptr_t at = (uintptr_t)m;  // the columns' common alignment
+  for (int c = 0; c < 4; c++) at |= (uintptr_t)a.c[c] | (uintptr_t)b.c[c];
+  if (a.layout == GVX_SOA && b.layout == GVX_SOA && at % 16 == 0)
+    mass_f32_x4_kernel<<<balanced_grid_of<mass_f32_x4_kernel>(threads, 0, n, 4 * threads), threads, 0, s>>>(
+        a, b, mo, n);
+  else if (a.layout == GVX_SOA && b.layout == GVX_SOA)
     mass_kernel<T, GVX_SOA, GVX_SOA>
         <<<balanced_grid_of<mass_kernel<T, GVX_SOA, GVX_SOA>>(threads, 0, n), threads, 0, s>>>(a, b, mo, n);
   else if (a.layout == GVX_SOA)
