@@ -26,7 +26,7 @@
 //
 // Bound by issue and the shared-memory/L1 data pipe together (430 warp instructions and 115 data
 // wavefronts per 32 pairs, of which the two table gathers take about 40).  2^20 events, 33.5 M
-// pairs: 0.582 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
+// pairs: 0.564 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
 // and a search per pair (620 instructions per 32 pairs, FP64 pipe 35% busy).  Six CTAs of 128
 // threads per SM (80 registers): eight (64 registers, 0.623 ms) leave the tables too little L1.
 // Tiles of 64 events on 128 threads: 0.615 ms; 256 on 256: 0.587 ms.
@@ -54,22 +54,36 @@ constexpr unsigned long long kMaxPolls = 1ull << 26;        // backstop if the t
 constexpr size_t kWsHeader = 256;                           // tile counter, padded
 constexpr int kMinTE = 64;
 
-// Staged particles: of one batch of a warp, or of one event by the CTA.
+// Staged particles: of one batch of a warp, or of one event by the CTA.  An array per member: the
+// lanes of a pair loop read neighbouring partners, and whole records 64 bytes apart put four of them on
+// the same banks (0.583 ms).
 struct Staged {
-  ffm::EvPart *part;
+  float4 *dy;       // (D.hi, Y.hi, D.lo, Y.lo)
+  longlong2 *ang;   // (eta, phi), units of 2^-59
   float4 *c0, *c1;  // (px, py) and (pz, E): float-float as (hi, hi, lo, lo), or two doubles
+  float2 *pt;
+  uint32_t *scale;  // the event's scale field, or 0: outside the float-float domain
+  __device__ __forceinline__ ffm::EvPart part(int c) const {
+    const longlong2 a = ang[c];
+    const float2 t = pt[c];
+    return ffm::EvPart{dy[c], a.x, a.y, t.x, t.y, scale[c], 0u};
+  }
 };
+constexpr size_t kStagedBytes = 3 * sizeof(float4) + sizeof(longlong2) + sizeof(float2) + sizeof(uint32_t);
 
 // One warp's part of shared memory.
 struct __align__(16) WarpBuf {
-  ffm::EvPart part[kCapW];
+  float4 dy[kCapW];
+  longlong2 ang[kCapW];
   float4 c0[kCapW], c1[kCapW];
+  float2 pt[kCapW];
+  uint32_t sc[kCapW];
   int4 info[32];  // by non-empty event: first particle, particles, first pair, event of the tile
   uint32_t scale[32];  // by non-empty event: the largest high word of pt and |m|
   int row[kCapW];      // by row: its particle, and what turns a pair's index into the partner
   uint32_t rows[kRows];  // bit q: a row starts at pair q of the batch
 };
-static_assert(4 * sizeof(WarpBuf) >= (size_t)kCP * (sizeof(ffm::EvPart) + 2 * sizeof(float4)),
+static_assert(4 * sizeof(WarpBuf) >= (size_t)kCP * kStagedBytes,
               "an event staged by the CTA takes the place of four warps' buffers");
 
 struct JArgs {
@@ -171,7 +185,10 @@ __device__ __forceinline__ bool stage_particle(const Staged &S, int c, const V4<
     const ffm::ff re = ffm::fx_half_reduce(2 * ae, &n), rp = ffm::fx_half_reduce(2 * ap, &j);
     ffm::ff sh, sn, cs;
     const ffm::LcLeg<ffm::ff> L = ffm::lc_leg_at(ptf, mmf, re, &n, T.hyp, &sh);
-    S.part[c] = ffm::EvPart{make_float4(L.D.hi, L.Y.hi, L.D.lo, L.Y.lo), ae, ap, ptf.hi, ptf.lo, ew, 0u};
+    S.dy[c] = make_float4(L.D.hi, L.Y.hi, L.D.lo, L.Y.lo);
+    S.ang[c] = make_longlong2(ae, ap);
+    S.pt[c] = make_float2(ptf.hi, ptf.lo);
+    S.scale[c] = ew;
     ffm::sincos_lc_at(rp, j, T.sin, &sn, &cs);
     const float sphi = (ffm::dhi(phi) >> 31) ? -1.0f : 1.0f, seta = (ffm::dhi(eta) >> 31) ? -1.0f : 1.0f;
     const ffm::ff px = ffm::lc_mul(ptf, cs), py = ffm::lc_scale(ffm::lc_mul(ptf, sn), sphi);
@@ -181,7 +198,7 @@ __device__ __forceinline__ bool stage_particle(const Staged &S, int c, const V4<
     return true;
   }
   if constexpr (F64) cartesian_f64(x, reinterpret_cast<double2 *>(S.c0 + c), reinterpret_cast<double2 *>(S.c1 + c));
-  S.part[c].scale = 0u;
+  S.scale[c] = 0u;
   return false;
 }
 
@@ -189,14 +206,14 @@ __device__ __forceinline__ bool stage_particle(const Staged &S, int c, const V4<
 // particles in *f (lanes); with F64 also the FP64 terms of the others in d, and the result is the
 // event's scale field if any particle is on the fast path (otherwise that of the last particle).
 template <bool F64>
-__device__ __forceinline__ uint32_t sum_places(const float4 *col, const ffm::EvPart *part, int c, int end,
+__device__ __forceinline__ uint32_t sum_places(const float4 *col, const uint32_t *scale, int c, int end,
                                                int step, ffm::ff2 *f, double *d) {
   ffm::ff2 a = {ffm::bc2(0.0f), ffm::bc2(0.0f)};
   uint32_t ew = 0;
   d[0] = d[1] = 0.0;
   for (; c < end; c += step) {
     const float4 v = col[c];
-    const uint32_t w = F64 ? part[c].scale : 1u;
+    const uint32_t w = F64 ? scale[c] : 1u;
     if (w) {
       a = ffm::add_same(a, ffm::ff2{ffm::mk2(v.x, v.y), ffm::mk2(v.z, v.w)});
       ew = w;
@@ -206,7 +223,7 @@ __device__ __forceinline__ uint32_t sum_places(const float4 *col, const ffm::EvP
       d[1] += r.y;
     }
   }
-  if constexpr (!F64) ew = part[end - 1].scale;
+  if constexpr (!F64) ew = scale[end - 1];
   *f = a;
   return ew;
 }
@@ -238,7 +255,7 @@ __device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, W
                                           int64_t base) {
   const int lane = threadIdx.x & 31;
   const unsigned upto = 0xffffffffu >> (31 - lane), below = upto >> 1;
-  const Staged S = {W.part, W.c0, W.c1};
+  const Staged S = {W.dy, W.ang, W.c0, W.c1, W.pt, W.sc};
   const int64_t pb = __shfl_sync(kAll, lo, 0);
   const int np = (int)(__shfl_sync(kAll, hi, take - 1) - pb);
   const int64_t q0 = s_pp[sb];
@@ -297,7 +314,7 @@ __device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, W
       const int h = (t >> 1) & 1;
       ffm::ff2 f;
       double d[2];
-      uint32_t ew = sum_places<RARE>(h ? S.c1 : S.c0, S.part, v.x + (t & 1), v.x + v.y, 2, &f, d);
+      uint32_t ew = sum_places<RARE>(h ? S.c1 : S.c0, S.scale, v.x + (t & 1), v.x + v.y, 2, &f, d);
       const unsigned pair = 3u << (lane & 30);
       const ffm::ff2 g = {ffm::mk2(__shfl_xor_sync(pair, f.hi.x, 1), __shfl_xor_sync(pair, f.hi.y, 1)),
                           ffm::mk2(__shfl_xor_sync(pair, f.lo.x, 1), __shfl_xor_sync(pair, f.lo.y, 1))};
@@ -325,7 +342,7 @@ __device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, W
       const int rec = W.row[rows + __popc(w & upto)];
       const int i = rec & 0xff, j = q + (rec >> 8);
       if (GVX_IN_BOUNDS(i, np, A.status) && GVX_IN_BOUNDS(j, np, A.status)) {
-        const ffm::EvPart &a = W.part[i], &b = W.part[j];
+        const ffm::EvPart a = S.part(i), b = S.part(j);
         ffm::ff m2s;
         const bool ok = !(extreme && (a.scale == 0u || b.scale == 0u)) && ffm::ev_pair_m2(a, b, T, &m2s);
         if constexpr (RARE) {
@@ -389,7 +406,7 @@ __device__ __forceinline__ bool staged_event(const JArgs &A, const ffm::LcTab &T
   if (threadIdx.x < 2) {
     ffm::ff2 f;
     double d[2];
-    const uint32_t ew = sum_places<true>(threadIdx.x ? S.c1 : S.c0, S.part, 0, n, 1, &f, d);
+    const uint32_t ew = sum_places<true>(threadIdx.x ? S.c1 : S.c0, S.scale, 0, n, 1, &f, d);
     put_sums<LS>(A, e, threadIdx.x, sum_to_double(ffm::lane_x(f), ew, d[0]), sum_to_double(ffm::lane_y(f), ew, d[1]));
   }
   const int total = n * (n - 1) / 2;
@@ -402,7 +419,7 @@ __device__ __forceinline__ bool staged_event(const JArgs &A, const ffm::LcTab &T
       fits = false;
       continue;
     }
-    const ffm::EvPart &a = S.part[i], &b = S.part[j];
+    const ffm::EvPart a = S.part(i), b = S.part(j);
     ffm::ff m2s;
     if (a.scale != 0u && b.scale != 0u && ffm::ev_pair_m2(a, b, T, &m2s))
       st_s(A.pair_m + out0 + q, ffm::lc_mass_out(m2s, a.scale));
@@ -424,9 +441,12 @@ __device__ __noinline__ void finish_tile(const JArgs &A, unsigned char *s_dyn, i
                                 base, &large);
   __syncthreads();
   Staged S;
-  S.part = reinterpret_cast<ffm::EvPart *>(s_dyn);
-  S.c0 = reinterpret_cast<float4 *>(S.part + kCP);
+  S.dy = reinterpret_cast<float4 *>(s_dyn);
+  S.ang = reinterpret_cast<longlong2 *>(S.dy + kCP);
+  S.c0 = reinterpret_cast<float4 *>(S.ang + kCP);
   S.c1 = S.c0 + kCP;
+  S.pt = reinterpret_cast<float2 *>(S.c1 + kCP);
+  S.scale = reinterpret_cast<uint32_t *>(S.pt + kCP);
   for (int e = 0; e < ne; e++) {
     const int64_t pb = s_off[e], n = s_off[e + 1] - pb;
     if (n <= kCapW) continue;
