@@ -26,7 +26,7 @@
 //
 // Bound by issue and the shared-memory/L1 data pipe together (430 warp instructions and 115 data
 // wavefronts per 32 pairs, of which the two table gathers take about 40).  2^20 events, 33.5 M
-// pairs: 0.564 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
+// pairs: 0.558 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
 // and a search per pair (620 instructions per 32 pairs, FP64 pipe 35% busy).  Six CTAs of 128
 // threads per SM (80 registers): eight (64 registers, 0.623 ms) leave the tables too little L1.
 // Tiles of 64 events on 128 threads: 0.615 ms; 256 on 256: 0.587 ms.
@@ -56,7 +56,7 @@ constexpr int kMinTE = 64;
 
 // Staged particles: of one batch of a warp, or of one event by the CTA.  An array per member: the
 // lanes of a pair loop read neighbouring partners, and whole records 64 bytes apart put four of them on
-// the same banks (0.583 ms).
+// the same banks (0.583 ms; 0.564 ms so).
 struct Staged {
   float4 *dy;       // (D.hi, Y.hi, D.lo, Y.lo)
   longlong2 *ang;   // (eta, phi), units of 2^-59
@@ -361,25 +361,35 @@ __device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, W
   return (lim < total ? kOver : 0) | (rare || extreme ? kRare : 0);
 }
 
-// The tile's batches, every warp walking the tile and taking its turn; *large: an event was left
-// to the CTA.
+// The tile's batches, every warp walking the tile: in the first walk a warp that ends a batch draws the
+// number of its next one from *next (their costs differ, and fixed turns leave warps waiting at the
+// tile's end: 0.564 ms), in the second they take turns.  *large: an event was left to the CTA.
 template <int NT, int LP, int LS, bool RARE>
 __device__ __forceinline__ int walk_tile(const JArgs &A, const ffm::LcTab &T, WarpBuf &W, int64_t e0,
                                          int ne, const int64_t *s_off, const int64_t *s_pp, int64_t base,
-                                         bool *large) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int seen = 0;
-  for (int sb = 0, turn = 0; sb < ne;) {
+                                         int *next, bool *large) {
+  const int lane = threadIdx.x & 31;
+  int seen = 0, mine = threadIdx.x >> 5;
+  for (int sb = 0, number = 0; sb < ne; number++) {
     const int64_t lo = s_off[min(sb + lane, ne)], hi = s_off[min(sb + lane + 1, ne)];
     const int64_t pb = __shfl_sync(kAll, lo, 0);
     const int take = __popc(__ballot_sync(kAll, sb + lane < ne && hi - pb <= kCapW));
     if (take == 0) {
       *large = true;
       sb++;
+      number--;
       continue;
     }
-    if (turn == warp) seen |= warp_batch<LP, LS, RARE>(A, T, W, e0, sb, take, lo, hi, s_pp, base);
-    turn = turn + 1 == NT / 32 ? 0 : turn + 1;
+    if (number == mine) {
+      seen |= warp_batch<LP, LS, RARE>(A, T, W, e0, sb, take, lo, hi, s_pp, base);
+      if constexpr (RARE) {
+        mine += NT / 32;
+      } else {
+        int t = 0;
+        if (lane == 0) t = atomicAdd(next, 1);
+        mine = __shfl_sync(kAll, t, 0);
+      }
+    }
     sb += take;
   }
   return seen;
@@ -438,7 +448,7 @@ __device__ __noinline__ void finish_tile(const JArgs &A, unsigned char *s_dyn, i
   bool large;
   if (rare)
     walk_tile<NT, LP, LS, true>(A, T, reinterpret_cast<WarpBuf *>(s_dyn)[threadIdx.x >> 5], e0, ne, s_off, s_pp,
-                                base, &large);
+                                base, nullptr, &large);
   __syncthreads();
   Staged S;
   S.dy = reinterpret_cast<float4 *>(s_dyn);
@@ -507,11 +517,15 @@ __global__ void __launch_bounds__(NT, 768 / NT) event_pairs_kernel(const __grid_
   __shared__ int64_t s_warp[NT / 32];
   __shared__ int64_t s_base;
   __shared__ int64_t s_tile;
+  __shared__ int s_next;
   const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   for (;;) {
-    if (threadIdx.x == 0) s_tile = (int64_t)atomicAdd(A.counter, 1u);
+    if (threadIdx.x == 0) {
+      s_tile = (int64_t)atomicAdd(A.counter, 1u);
+      s_next = NT / 32;
+    }
     __syncthreads();
     const int64_t tile = s_tile;
     if (tile >= A.n_tiles) break;
@@ -555,7 +569,8 @@ __global__ void __launch_bounds__(NT, 768 / NT) event_pairs_kernel(const __grid_
 
     // 3. the batches, 4. what they leave
     bool large = false;
-    const int seen = walk_tile<NT, LP, LS, false>(A, T, bufs[warp], e0, ne, s_off, s_pp, base, &large);
+    const int seen = walk_tile<NT, LP, LS, false>(A, T, bufs[warp], e0, ne, s_off, s_pp, base, &s_next,
+                                                        &large);
     if ((seen & kOver) && lane == 0) raise_status(A.status, GVX_ERR_CAPACITY);
     const bool rare = __syncthreads_or(seen & kRare);
     if (rare || large) finish_tile<NT, LP, LS>(A, s_dyn, e0, ne, s_off, s_pp, base, rare);
