@@ -241,11 +241,10 @@ gvx_status gvx_event_pair_masses(const gvx_lv *particles, const int64_t *offsets
  * Deterministic (a fixed summation order per particle).  Offsets or pair offsets that do not
  * match the event sizes or n_pairs are detected on the device: GVX_ERR_OFFSETS is recorded in the
  * device status word and the gradients of the affected events are not written.  All pointers
- * are device (or GPU-addressable host) memory; nothing is allocated.  One 8-byte memset and two
- * launches: the staged float-float pass, which lists in the workspace the tiles of 14 events
- * that met a rare FP64 case (a pair or event-sum part outside the float-float domain, an event
- * of more than 128 particles or 640 pairs), then a pass over the listed tiles alone that adds
- * those contributions (with none listed it returns at once).
+ * are device (or GPU-addressable host) memory; nothing is allocated.  Two launches: the staged
+ * float-float pass, which notes in the workspace what it left of each tile of events (pairs and
+ * event-sum parts outside the float-float domain, events of more than 64 particles), then a pass
+ * over the tiles noted alone that adds those contributions (with none it returns at once).
  */
 gvx_status gvx_event_pair_masses_bwd(const gvx_lv *particles, const int64_t *offsets,
                                      const int64_t *pair_offsets, int64_t n_events,

@@ -107,5 +107,15 @@ GVX_HD bool ev_pair_m2(const EvPart &a, const EvPart &b, const LcTab &T, ff *m2s
   return ok && (m2s->hi >= 8.27180613e-25f || m2s->hi == 0.0f);  // 2^-80
 }
 
+// Whether a staged angle is the FP64 one exactly: its last bit is at least 2^-59 from 2^-7 on.
+GVX_HD bool fx_exact(int64_t a) { return (a < 0 ? -a : a) >= (1ll << 52) || a == 0; }
+
+// Whether a pair's angle differences are exact (no angle below 2^-7, no turn taken off d_phi): then
+// S is good below kFxMinS too, and a launch seldom leaves a pair (one near pair in a hundred).
+GVX_HD bool ev_near_exact(const EvPart &a, const EvPart &b) {
+  const int64_t dp = a.phi - b.phi;
+  return fx_exact(a.eta) && fx_exact(b.eta) && fx_exact(a.phi) && fx_exact(b.phi) && wrap_fx(dp) == dp;
+}
+
 }  // namespace ffm
 }  // namespace gvx

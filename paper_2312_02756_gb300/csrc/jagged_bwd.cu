@@ -7,70 +7,74 @@
 //   grad_i = sum over j != i of gm[pair(i, j)] dm(p_i, p_j)/dp_i  +  J_i^T gs[e],
 // J_i = d(px, py, pz, E)/d(pt, eta, phi, m) of the particle.
 //
-// Pair part in light-cone form (mass_lc_grad.cuh): with Y = E + P, D = E - P = m^2/Y,
-// F = m^2 = (D_i + D_j)(Y_i + Y_j) + 4 pt_i pt_j S and c_ij = gm_ij / (2 m_ij),
-//   dm/dpt_i  = (cosh eta_i / E_i) (Y_i A1 - D_i A2) + 4 A5,
-//   dm/deta_i = (pt_i sinh eta_i / E_i) (Y_i A1 - D_i A2) + pt_i A6,
-//   dm/dphi_i = pt_i A7,
-//   dm/dm_i   = (2 m_i / E_i) (E_i A3 + A4),
-// summed over the partners j through seven accumulators (float-float sums whose absolute error
-// stays within ~2^-47 of the summed magnitudes)
-//   A1 = sum c D_j,  A2 = sum c Y_j,  A3 = sum c,  A4 = sum c E_j,  A5 = sum c pt_j S_ij,
-//   A6 = sum c pt_j 2 sinh(eta_i - eta_j),  A7 = sum c pt_j 2 sin(phi_i - phi_j),
-// so that a pair costs its angular terms and its mass once and each direction seven float-float
-// multiply-accumulates (paired FP32 lanes where two share a factor).
+// CTAs take tiles of consecutive events (grid-stride over tiles) and deal a tile's events to their
+// warps in batches of whole events of at most kCapW particles, as the forward kernel (jagged.cu)
+// does; a warp that ends a batch draws the next one's number.  Per batch, one warp, with its own
+// part of shared memory and no block barrier:
+//   (a) per particle: its light-cone terms at its event's power of two and its angles in fixed point
+//       (event_lc.cuh);
+//   (b) in chunks of kPC pairs, one lane per pair: the five numbers of event_lc_grad.cuh, which
+//       enter both legs' gradients with a sign only, into the pair's slot.  The pairs are taken by
+//       their distance: row t of an event of n particles holds the pairs (i, i + t modulo n);
+//   (c) after each chunk, one lane per particle: its signed sums over its pairs of the chunk, two per
+//       row, in a fixed order, so that the result does not depend on scheduling and no atomic
+//       operation touches it.  With the pairs in that order the lanes of an event read
+//       neighbouring slots;
+//   (d) per particle: its gradient from the sums, and J^T gs, both in float-float, converted by
+//       integer operations and added in FP64.
+// What that leaves is noted in a word per tile in the workspace and done by a second launch: pairs
+// outside the float-float domain (either particle outside the forward's domain at the event's scale
+// or with pt = 0, near-equal directions whose difference is not exact, a scaled m^2 below 2^-80, |gm|
+// outside [2^-60, 2^20]) and event-sum parts with gs out of range, by walking the batches that met one
+// once more and adding the FP64 formulas to the gradients written; and events with more than kCapW
+// particles, by a CTA straight from global memory with the elementwise adjoint.  The pair offsets
+// are those the forward call wrote; each tile checks them (and the offsets) against the event sizes
+// and the pair count before it reads any pair gradient, and records GVX_ERR_OFFSETS for a tile that
+// does not match (its particles' gradients are then not written).
 //
-// CTAs take tiles of kTE consecutive events (grid-stride over tiles) and stage them in
-// sub-batches of whole events of at most kNT particles and kPC pairs: (a) the raw particles, and
-// the order of the sub-batch's events by decreasing size (so that the lanes of a warp walk
-// partner loops of similar length); (b) per particle, by the thread that will take it in (d),
-// its event's scale and light-cone terms (at the event's scale, as the forward kernel stages
-// them) and its event-sum part J^T gs (float-float, in double in the thread's own shared-memory
-// slot); (c) one thread per pair: the pair's angular terms, m and c once, stored per pair as
-// c, c S and c (2 sinh d_eta, 2 sin d_phi); (d) one thread per particle walks its partners in a
-// fixed order, adding the seven sums from the pair slots and the partners' staged terms, and
-// assembles and converts its gradient -- so the result does not depend on scheduling and no
-// atomic operation touches it.  Pairs outside the float-float domain (either particle outside the
-// forward's domain at the event scale, |d_phi|/2 within 2^-7 of pi, a scaled m^2 below 2^-80,
-// |gm| outside [2^-60, 2^20]) are marked in (c) and take the FP64 formulas; so does an event-sum
-// part whose gs lies outside the float-float range, and an event with more than kNT particles or
-// kPC pairs is handled alone, straight from global memory, with the elementwise kernels' pair
-// adjoint.  These rare FP64 paths run in a second launch of the same kernel (FIX = true): the
-// first launch contains no function call (a call site costs the staged path ~12% in spills at
-// 96 registers), skips them and appends each tile that met one to a list in the caller's
-// workspace; the second launch takes only the listed tiles (none: it returns at once), repeats
-// their staging and classification and adds, per particle, the FP64 contributions to the
-// gradient the first launch wrote (big events it writes whole).  The pair offsets are
-// those the forward call wrote; each tile checks them (and the offsets) against the event sizes
-// and the pair count before it reads any pair gradient, and records GVX_ERR_OFFSETS for a tile
-// that does not match (its particles' gradients are then not written).
+// Bound by issue (the first launch; 58% of the slots, held back by dependent chains at 20 warps per SM).
+// 300,007 events, 9.6 M pairs: 382 us both launches, against 550 us for block-wide sub-batches whose
+// particles walked their partners (seven sums of products per direction, 1,150 warp instructions per
+// 32 pairs) and a second launch over every tile with a pair near 2 pi.  By step: pairs in packed
+// order, whose lanes read slots far apart, 465 us; by distance 413; without a call in the first
+// launch 392; chunks of 96 pairs and 5 CTAs per SM in place of 128 and 4 382 (64 pairs: 410).  Both
+// particles of a lane on paired FP32 instructions in (d): 422 us (moves and spills).
 #include <cuda_runtime.h>
 
-#include <limits.h>
-
 #include "common.cuh"
-#include "mass_lc_grad.cuh"
-#include "pair_index.cuh"
+#include "event_lc_grad.cuh"
 #include "pair_math.cuh"
 
 namespace gvx {
 namespace {
 
-constexpr int kTE = 14;    // events per tile (about 112 particles at the benchmark multiplicity)
-constexpr int kNT = 128;   // threads per CTA, and particles staged per sub-batch
-constexpr int kPC = 640;   // pairs staged per sub-batch (the events of a sub-batch average ~450)
-constexpr int kNoFast = INT_MIN;  // scale marker of a particle outside the float-float domain
-constexpr uint32_t kSlowPair = 0x7fc00000u;  // the bits of c.hi marking a pair for FP64
-// Workspace: the count of listed tiles (zeroed by the call before the first launch), then from
-// byte kWsList the list of tiles (int64) the FIX launch takes, at most one entry per tile.
-constexpr size_t kWsList = 256;
-// per staged particle: pt, eta, phi, m and the FP64 accumulator (doubles); (pt, Y), (D, E),
-// (cosh, sinh) (float4) and m (float2); the larger high word of pt and |m|, and its event's scale
-// field or kNoFast (ints); per staged pair: (c, c S) and (c 2 sinh d_eta, c 2 sin d_phi) (float4)
-constexpr size_t kDynSmem =
-    (size_t)kNT * (4 * sizeof(double) + sizeof(double4) + 3 * sizeof(float4) + sizeof(float2) +
-                   2 * sizeof(int)) +
-    (size_t)kPC * 2 * sizeof(float4);
+constexpr int kNT = 128;    // threads per CTA
+constexpr int kCtas = 5;    // CTAs per SM
+constexpr int kTE = 128;    // events per tile at most
+constexpr int kCapW = 64;   // particles per warp batch
+constexpr int kPC = 96;     // pairs per chunk
+constexpr int kRows = kCapW * (kCapW - 1) / 2 / 32 + 1;  // words of the row mask: a bit per pair
+constexpr unsigned kAll = 0xffffffffu;
+constexpr int kMinTE = 16;  // events per tile at least
+constexpr int kWsEvents = 14;  // gvx_event_pair_masses_bwd_workspace: a word per kWsEvents events
+static_assert(kMinTE >= kWsEvents, "the workspace holds a word per tile");
+
+// One warp's part of shared memory.
+struct __align__(16) WarpBuf {
+  float4 dy[kCapW];       // (D.hi, Y.hi, D.lo, Y.lo)
+  longlong2 ang[kCapW];   // (eta, phi), units of 2^-59
+  float4 w0[kPC], w1[kPC];  // by pair of the chunk: lanes (W, Ve) and (Z, U); in a second walk the
+  float2 w2[kPC];           // FP64 gradients by particle.  w2: Vp
+  float2 pt[kCapW];       // pt; hi < 0: outside the float-float domain
+  float2 mm[kCapW];       // m
+  float2 sum[5][kCapW];   // W, Ve, Z, U, Vp summed over the chunks so far
+  int4 info[32];          // by non-empty event: first particle, particles, first pair, event of the tile | first row << 8
+  uint32_t scale[32];     // by non-empty event: the largest high word of pt and |m|
+  int row[kCapW / 2];     // by row: its first pair, its event's first particle and size, the distance
+  uint32_t rows[kRows];   // bit q: a row starts at pair q of the batch
+};
+static_assert(sizeof(float4) * 2 * kPC >= sizeof(V4<double>) * kCapW, "FP64 gradients in place of the slots");
+constexpr size_t kDynSmem = (kNT / 32) * sizeof(WarpBuf);
 
 struct BArgs {
   Lv p;
@@ -81,8 +85,9 @@ struct BArgs {
   bool has_gsum;
   LvOut grad;
   int32_t *status;
-  unsigned long long *fix_count;  // workspace: tiles listed for the FIX launch
-  int64_t *fix_tiles;             // workspace: their indices
+  unsigned long long *left;  // workspace: a word per tile, what the first launch left of it
+  int te;   // events per tile
+  int cap;  // particles per batch (an event larger than it, up to kCapW, is a batch of its own)
 };
 
 // J^T gs in FP64 for one particle: gs = (gx, gy, gz, gE) against the rows
@@ -114,48 +119,6 @@ __device__ __noinline__ V4<double> sum_part(V4<double> x, V4<double> gs) {
   return g;
 }
 
-// The same J^T gs in float-float from the particle's staged light-cone terms (scaled by 2^-s:
-// pt, P, E, m; cosh and sinh of |eta|), gs converted at its own scale 2^sg; returned in double.
-// False when gs has a nonzero component outside [2^-300, 2^300] (the caller then uses sum_part).
-__device__ __forceinline__ bool sum_part_lc(ffm::ff pt, ffm::ff E, ffm::ff mm, ffm::ff ch,
-                                            ffm::ff sh, double eta, double phi, double m,
-                                            uint32_t eoff_s, V4<double> gs, const ffm::LcTab &T,
-                                            V4<double> *out) {
-  using namespace ffm;
-  const uint32_t h0 = dhi(gs.x) & 0x7fffffffu, h1 = dhi(gs.y) & 0x7fffffffu;
-  const uint32_t h2 = dhi(gs.z) & 0x7fffffffu, h3 = dhi(gs.w) & 0x7fffffffu;
-  const uint32_t hmax = umax32(umax32(h0, h1), umax32(h2, h3));
-  if (hmax == 0u && (dlo(gs.x) | dlo(gs.y) | dlo(gs.z) | dlo(gs.w)) == 0u) {
-    *out = V4<double>{0.0, 0.0, 0.0, 0.0};
-    return true;
-  }
-  if (hmax - (723u << 20) >= (600u << 20)) return false;  // scale field 723..1322
-  const uint32_t ewg = hmax & 0x7ff00000u, rbg = ewg - (127u << 20);
-  const ff gx = cvt1(cvt_parts(h0, dlo(gs.x), rbg)), gy = cvt1(cvt_parts(h1, dlo(gs.y), rbg));
-  const ff gz = cvt1(cvt_parts(h2, dlo(gs.z), rbg)), gE = cvt1(cvt_parts(h3, dlo(gs.w), rbg));
-  const float sx = sign_of(gs.x), sy = sign_of(gs.y), sz = sign_of(gs.z), sE = sign_of(gs.w);
-  const float seta = sign_of(eta), sphi = sign_of(phi), sm = sign_of(m);
-  ff sn, cs;  // sin and cos of |phi|
-  sincos_lc(cvt1(cvt_parts(dhi(phi) & 0x7fffffffu, dlo(phi), kRebaseOne)), T.sin, &sn, &cs);
-  const ff P = lc_mul(pt, ch);
-  const ff rE = lc_div(ff{1.0f, 0.0f}, E);
-  const ff e0 = lc_mul(lc_mul(P, ch), rE);           // dE/dpt
-  const ff e1 = lc_mul(lc_mul(P, lc_mul(pt, sh)), rE);  // |dE/deta| (times 2^-s)
-  const ff e3 = lc_mul(mm, rE);                       // |dE/dm|
-  // signed products (the sign of a product of signed values, on the hi and lo parts)
-  const auto sp = [](const ff &a, const ff &b, float sgn) { return lc_scale(lc_mul(a, b), sgn); };
-  const ff dpt = add_same(add_same(sp(gx, cs, sx), sp(gy, sn, sy * sphi)),
-                     add_same(sp(gz, sh, sz * seta), sp(gE, e0, sE)));
-  const ff deta = add_same(sp(gz, P, sz), sp(gE, e1, sE * seta));
-  const ff dphi = lc_mul(pt, add_same(sp(gy, cs, sy), sp(gx, sn, -sx * sphi)));
-  const ff dm = sp(gE, e3, sE * sm);
-  const uint32_t eoff_g = ewg - (127u << 20);       // 2^sg
-  const uint32_t eoff_gs = eoff_g + eoff_s - (896u << 20);  // 2^(sg + s)
-  *out = V4<double>{lc_to_double(dpt, eoff_g), lc_to_double(deta, eoff_gs),
-                    lc_to_double(dphi, eoff_gs), lc_to_double(dm, eoff_g)};
-  return true;
-}
-
 // gm-weighted gradient of particle i's leg over its partners in one event, everything read from
 // global memory (the path of events too large to stage).
 template <int LP>
@@ -182,11 +145,10 @@ __device__ __forceinline__ void partners_from_global(const BArgs &A, const ffm::
   }
 }
 
-// An event with more than kNT particles (rare): its particles in strides of the CTA, each
-// against all its partners from global memory.  Out of line, so that its registers do not count
-// against the staged path's.
+// An event with more than kCapW particles: its particles in strides of the CTA, each against all its
+// partners from global memory.
 template <int LP, int LS, int LG>
-__device__ __noinline__ void big_event(const BArgs &A, const ffm::LcTab &T, int64_t e, int64_t pbeg,
+__device__ __forceinline__ void big_event(const BArgs &A, const ffm::LcTab &T, int64_t e, int64_t pbeg,
                                        int64_t n, int64_t pair0) {
   for (int64_t t = threadIdx.x; t < n; t += kNT) {
     double acc[4] = {0.0, 0.0, 0.0, 0.0};
@@ -203,349 +165,451 @@ __device__ __noinline__ void big_event(const BArgs &A, const ffm::LcTab &T, int6
   }
 }
 
-// One pair outside the float-float domain: its FP64 gradient of the first leg added to *slot.
-__device__ __noinline__ void slow_pair_add(V4<double> x, V4<double> y, double g, double4 *slot) {
-  V4<double> g1, g2;
-  pair_mass_grad(x, y, g, g1, g2);
-  double4 a = *slot;
-  a.x += g1.x;
-  a.y += g1.y;
-  a.z += g1.z;
-  a.w += g1.w;
-  *slot = a;
+// (a) The particles of places c and c + 32 (the second only with `two`) at their events' scale words,
+// as the lanes of paired FP32 instructions.  False where one lies outside the float-float domain.
+__device__ __forceinline__ bool stage_particles(WarpBuf &W, int c, bool two, const V4<double> *x,
+                                                const uint32_t *wmax, const ffm::LcTab &T) {
+  bool ok[2];
+  ffm::ff pt[2], mm[2], re[2];
+  int64_t ae[2], ap[2];
+  uint32_t n[2];
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const uint32_t hp = ffm::dhi(x[r].x), hm = ffm::dhi(x[r].w) & 0x7fffffffu;
+    ok[r] = hp >= 0x100000u && ffm::lc_in_domain(hp, hm, ffm::dhi(x[r].y) & 0x7fffffffu,
+                                                 ffm::dhi(x[r].z) & 0x7fffffffu, wmax[r]);
+    const uint32_t rb = (wmax[r] & 0x7ff00000u) - (127u << 20);
+    pt[r] = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(x[r].x), rb));
+    mm[r] = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(x[r].w), rb));
+    ae[r] = ffm::angle_fx(x[r].y);
+    ap[r] = ffm::angle_fx(x[r].z);
+    re[r] = ffm::fx_half_reduce(2 * ae[r], &n[r]);
+  }
+  const ffm::LcLeg<ffm::ff2> L =
+      ffm::lc_leg_at(ffm::pack(pt[0], pt[1]), ffm::pack(mm[0], mm[1]), ffm::pack(re[0], re[1]), n, T.hyp);
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    if (r == 1 && !two) break;
+    const int k = c + 32 * r;
+    const ffm::ff D = r ? ffm::lane_y(L.D) : ffm::lane_x(L.D), Y = r ? ffm::lane_y(L.Y) : ffm::lane_x(L.Y);
+    const ffm::ff ms = ffm::with_sign(mm[r], ffm::dhi(x[r].w));
+    W.dy[k] = make_float4(D.hi, Y.hi, D.lo, Y.lo);
+    W.ang[k] = make_longlong2(ae[r], ap[r]);
+    W.pt[k] = make_float2(ok[r] ? pt[r].hi : -1.0f, pt[r].lo);
+    W.mm[k] = make_float2(ms.hi, ms.lo);
+  }
+  return ok[0] && (ok[1] || !two);
 }
 
-__device__ __forceinline__ float4 pack4(const ffm::ff &a, const ffm::ff &b) {
-  return make_float4(a.hi, a.lo, b.hi, b.lo);
+__device__ __forceinline__ ffm::EvPart staged(const WarpBuf &W, int c) {
+  const longlong2 a = W.ang[c];
+  const float2 t = W.pt[c];
+  return ffm::EvPart{W.dy[c], a.x, a.y, t.x, t.y, 0u, 0u};
 }
 
-template <int LP, int LS, int LG, bool FIX>
-__global__ void __launch_bounds__(kNT, 5) event_pairs_bwd_kernel(BArgs A) {
-  bool fix = false;  // FIX == false: this thread met an FP64 path in the current tile
-  using ffm::ff;
-  using ffm::ff2;
-  extern __shared__ double s_dyn[];
-  double *s_pt = s_dyn, *s_eta = s_pt + kNT, *s_phi = s_eta + kNT, *s_m = s_phi + kNT;
-  double4 *s_acc = reinterpret_cast<double4 *>(s_m + kNT);  // FP64 part of each gradient
-  float4 *s_pY = reinterpret_cast<float4 *>(s_acc + kNT);   // (pt, Y)
-  float4 *s_DE = s_pY + kNT;                                // (D, E)
-  float4 *s_cs = s_DE + kNT;                                // (cosh, sinh) of |eta|
-  float2 *s_mm = reinterpret_cast<float2 *>(s_cs + kNT);    // |m|
-  int *s_sc = reinterpret_cast<int *>(s_mm + kNT), *s_fs = s_sc + kNT;
-  float4 *s_w0 = reinterpret_cast<float4 *>(s_fs + kNT);  // per pair: (c, c S)
-  float4 *s_w1 = s_w0 + kPC;                              // (c 2 sinh d_eta, c 2 sin d_phi)
-  __shared__ int64_t s_off[kTE + 1], s_poff[kTE + 1];
-  __shared__ int s_order[kTE], s_start[kTE];
-  __shared__ int s_bad;
-  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
-  const int64_t n_tiles = (A.n_events + kTE - 1) / kTE;
-  // the first launch: every tile; the FIX launch: the listed ones (written by the first launch)
-  const int64_t n_iter = FIX ? (int64_t)*(volatile unsigned long long *)A.fix_count : n_tiles;
-  const int k = threadIdx.x;
-  for (int64_t it = blockIdx.x; it < n_iter; it += gridDim.x) {
-    int64_t tile = it;
-    if constexpr (FIX) {
-      tile = A.fix_tiles[it];
-      if (!GVX_IN_BOUNDS(tile, n_tiles, A.status)) continue;
+// a += x, the leading parts without error.
+__device__ __forceinline__ void acc_add(ffm::ff2 &a, const ffm::ff2 &x) {
+  const ffm::ff2 s = ffm::two_sum2(a.hi, x.hi);
+  a = {s.hi, ffm::add2(a.lo, ffm::add2(s.lo, x.lo))};
+}
+__device__ __forceinline__ void acc_add(ffm::ff &a, const ffm::ff &x) {
+  const ffm::ff s = ffm::two_sum(a.hi, x.hi);
+  a = {s.hi, ffm::fadd(a.lo, ffm::fadd(s.lo, x.lo))};
+}
+struct Sums {
+  ffm::ff2 we, zu;
+  ffm::ff vp;
+};
+__device__ __forceinline__ void add_slot(Sums &s, const WarpBuf &W, int k) {
+  const float4 a = W.w0[k], b = W.w1[k];
+  const float2 v = W.w2[k];
+  acc_add(s.we, ffm::ff2{ffm::mk2(a.x, a.y), ffm::mk2(a.z, a.w)});
+  acc_add(s.zu, ffm::ff2{ffm::mk2(b.x, b.y), ffm::mk2(b.z, b.w)});
+  acc_add(s.vp, ffm::ff{v.x, v.y});
+}
+
+// One batch by one warp: `take` events of the tile from event sb on (lane l < take having event
+// sb + l with particles lo .. hi - 1), together at most kCapW particles.  RARE: a second walk, which
+// adds what the first one left to the gradients written and nothing else.  Returns whether
+// something was left.
+template <int LP, int LS, int LG, bool RARE>
+__device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, WarpBuf &W, int64_t e0,
+                                           int sb, int take, int64_t lo, int64_t hi, const int64_t *s_po) {
+  const int lane = threadIdx.x & 31;
+  const unsigned upto = 0xffffffffu >> (31 - lane), below = upto >> 1;
+  const int64_t pb = __shfl_sync(kAll, lo, 0);
+  const int np = (int)(__shfl_sync(kAll, hi, take - 1) - pb);
+  const int64_t q0 = s_po[sb];
+  const int total = (int)(s_po[sb + take] - q0);
+  const double *const gpm = A.gpm + q0;
+  V4<double> x[2] = {{0.0, 0.0, 0.0, 0.0}, {0.0, 0.0, 0.0, 0.0}};
+#pragma unroll
+  for (int r = 0; r < 2; r++)
+    if (lane + 32 * r < np && GVX_IN_BOUNDS(pb + lane + 32 * r, A.n_particles, A.status))
+      x[r] = ld4c<LP>(A.p, pb + lane + 32 * r);
+  // non-empty events in order; the particles they start at as bits
+  const int n_l = lane < take ? (int)(hi - lo) : 0, st_l = (int)(lo - pb);
+  const unsigned nz = __ballot_sync(kAll, n_l > 0);
+  const unsigned m0 = __reduce_or_sync(kAll, n_l > 0 && st_l < 32 ? 1u << st_l : 0u);
+  const unsigned m1 = __reduce_or_sync(kAll, n_l > 0 && st_l >= 32 ? 1u << (st_l - 32) : 0u);
+  int nrow = n_l >> 1;  // rows up to and with the lane's event
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kAll, nrow, o);
+    if (lane >= o) nrow += t;
+  }
+  if (n_l > 0) {
+    const int k = __popc(nz & below);
+    W.info[k] = make_int4(st_l, n_l, (int)(s_po[sb + lane] - q0), (sb + lane) | (nrow - (n_l >> 1)) << 8);
+    W.scale[k] = 0u;
+  }
+  for (int w = lane; w < kRows; w += 32) W.rows[w] = 0u;
+  __syncwarp();
+  int rank[2];
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    rank[r] = r ? __popc(m0) + __popc(m1 & upto) - 1 : __popc(m0 & upto) - 1;
+    if (lane + 32 * r < np)
+      atomicMax(&W.scale[rank[r]], ffm::umax32(ffm::dhi(x[r].x), ffm::dhi(x[r].w) & 0x7fffffffu));
+  }
+  __syncwarp();
+  bool rare = false;
+  uint32_t wmax[2] = {0u, 0u};
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const int c = lane + 32 * r;
+    if (c < np) {
+      const int4 v = W.info[rank[r]];
+      const int li = c - v.x;
+      if (li > 0 && 2 * li <= v.y) {  // row li: pairs (i, i + li), i from 0, at slots first + i
+        const int first = v.z + (li - 1) * v.y;
+        W.row[(v.w >> 8) + li - 1] = first | v.x << 11 | v.y << 17 | li << 24;
+        atomicOr(&W.rows[first >> 5], 1u << (first & 31));
+      }
+      wmax[r] = W.scale[rank[r]];
     }
-    const int64_t e0 = tile * kTE;
-    const int ne = (int)(A.n_events - e0 < kTE ? A.n_events - e0 : kTE);
-    __syncthreads();  // the previous tile is done with the shared arrays
-    if (threadIdx.x == 0) s_bad = 0;
-    if (threadIdx.x <= ne) {
-      s_off[threadIdx.x] = A.off[e0 + threadIdx.x];
-      s_poff[threadIdx.x] = A.pair_off[e0 + threadIdx.x];
+  }
+  if (lane < np) rare = !stage_particles(W, lane, lane + 32 < np, x, wmax, T);
+  V4<double> *const dg = reinterpret_cast<V4<double> *>(W.w0);  // RARE: FP64 gradients by particle
+#pragma unroll
+  for (int r = 0; r < 2; r++) {
+    const int c = lane + 32 * r;
+    if constexpr (RARE) {
+      dg[c] = {0.0, 0.0, 0.0, 0.0};
+    } else {
+#pragma unroll
+      for (int k = 0; k < 5; k++) W.sum[k][c] = make_float2(0.0f, 0.0f);
     }
-    __syncthreads();
-    if (threadIdx.x < ne) {
-      const int64_t a = s_off[threadIdx.x], b = s_off[threadIdx.x + 1], n = b - a;
-      const int64_t pa = s_poff[threadIdx.x], pb = s_poff[threadIdx.x + 1];
-      bool bad = a < 0 || n < 0 || b > A.n_particles || n > (1ll << 31) || pa < 0 ||
-                 pb > A.n_pairs || pb - pa != n * (n - 1) / 2;
-      if (e0 + threadIdx.x == 0 && (a != 0 || pa != 0)) bad = true;
-      if (bad) s_bad = 1;
+  }
+  const bool extreme = __any_sync(kAll, rare);  // and the staged places are visible to the warp
+  int rows = -1;  // rows that start before the current word, less one
+  for (int c0 = 0; c0 < total; c0 += kPC) {
+    const int c1 = c0 + kPC < total ? c0 + kPC : total;
+    // (b)
+    for (int r0 = c0; r0 < c1; r0 += 32) {
+      const unsigned w = W.rows[r0 >> 5];
+      const int q = r0 + lane;
+      int i = 0, j = 0;
+      bool slow = false;
+      double g = 0.0;
+      if (q < c1) {
+        const int rec = W.row[rows + __popc(w & upto)];
+        const int first = rec & 0x7ff, base = (rec >> 11) & 0x3f, n = (rec >> 17) & 0x7f, t = rec >> 24;
+        i = q - first;
+        j = i + t < n ? i + t : i + t - n;
+        const int a = min(i, j);  // its number in the packed order
+        const int k = first - (t - 1) * n + a * n - (a * (a + 1) >> 1) + (max(i, j) - a - 1);
+        if (GVX_IN_BOUNDS(q0 + k, A.n_pairs, A.status)) g = __ldg(gpm + k);
+        i += base;
+        j += base;
+        if (GVX_IN_BOUNDS(i, np, A.status) && GVX_IN_BOUNDS(j, np, A.status)) {
+          const ffm::EvPart a = staged(W, i), b = staged(W, j);
+          ffm::EvGrad o;
+          slow = !ffm::ev_pair_grad(a, b, g, T, &o) || (extreme && (a.pt_hi < 0.0f || b.pt_hi < 0.0f));
+          if constexpr (!RARE) {
+            if (slow) {
+              o = ffm::EvGrad{{ffm::bc2(0.0f), ffm::bc2(0.0f)}, {ffm::bc2(0.0f), ffm::bc2(0.0f)}, {0.0f, 0.0f}};
+              rare = true;
+            }
+            W.w0[q - c0] = make_float4(o.we.hi.x, o.we.hi.y, o.we.lo.x, o.we.lo.y);
+            W.w1[q - c0] = make_float4(o.zu.hi.x, o.zu.hi.y, o.zu.lo.x, o.zu.lo.y);
+            W.w2[q - c0] = make_float2(o.vp.hi, o.vp.lo);
+          }
+        }
+      }
+      rows += __popc(w);
+      if constexpr (RARE) {  // the pairs left, their gradients added in the pairs' order
+        V4<double> g1 = {0, 0, 0, 0}, g2 = {0, 0, 0, 0};
+        if (slow) pair_mass_grad(ld4c<LP>(A.p, pb + i), ld4c<LP>(A.p, pb + j), g, g1, g2);
+        for (unsigned left = __ballot_sync(kAll, slow); left; left &= left - 1) {
+          if (lane == __ffs((int)left) - 1) {
+            V4<double> t = dg[i];
+            dg[i] = {t.x + g1.x, t.y + g1.y, t.z + g1.z, t.w + g1.w};
+            t = dg[j];
+            dg[j] = {t.x + g2.x, t.y + g2.y, t.z + g2.z, t.w + g2.w};
+          }
+          __syncwarp();
+        }
+      }
     }
-    __syncthreads();
-    if (s_bad) {
-      if (threadIdx.x == 0) raise_status(A.status, GVX_ERR_OFFSETS);
-      continue;
+    __syncwarp();
+    // (c)
+    if constexpr (!RARE) {
+#pragma unroll 1
+      for (int r = 0; r < 2; r++) {
+        const int c = lane + 32 * r;
+        if (c >= np) break;
+        const int4 v = W.info[r ? rank[1] : rank[0]];
+        const int n = v.y, li = c - v.x;
+        if (v.z >= c1 || v.z + (n * (n - 1) >> 1) <= c0) continue;
+        Sums s;
+        {
+          const float2 a = W.sum[0][c], b = W.sum[1][c], d = W.sum[2][c], e = W.sum[3][c], f = W.sum[4][c];
+          s.we = {ffm::mk2(a.x, b.x), ffm::mk2(a.y, b.y)};
+          s.zu = {ffm::mk2(d.x, e.x), ffm::mk2(d.y, e.y)};
+          s.vp = {f.x, f.y};
+        }
+        // row t: pair (li, li + t) at the row's place li, and (li - t, li) at place li - t, modulo n;
+        // the last row of an even n holds each of its n / 2 pairs once
+        Sums o = {{ffm::bc2(0.0f), ffm::bc2(0.0f)}, {ffm::bc2(0.0f), ffm::bc2(0.0f)}, {0.0f, 0.0f}};
+        const int len = c1 - c0;
+        int t = c0 > v.z ? (c0 - v.z) / n + 1 : 1;
+        for (int f = v.z + (t - 1) * n - c0; 2 * t <= n && f < len; t++, f += n) {
+          const int in = li >= t ? li - t : li - t + n, last = 2 * t == n ? t : n;
+          if (li < last && (unsigned)(f + li) < (unsigned)len) add_slot(s, W, f + li);
+          if (in < last && (unsigned)(f + in) < (unsigned)len) add_slot(o, W, f + in);
+        }
+        acc_add(s.we, ffm::neg(o.we));
+        acc_add(s.zu, o.zu);
+        acc_add(s.vp, ffm::neg(o.vp));
+        W.sum[0][c] = make_float2(s.we.hi.x, s.we.lo.x);
+        W.sum[1][c] = make_float2(s.we.hi.y, s.we.lo.y);
+        W.sum[2][c] = make_float2(s.zu.hi.x, s.zu.lo.x);
+        W.sum[3][c] = make_float2(s.zu.hi.y, s.zu.lo.y);
+        W.sum[4][c] = make_float2(s.vp.hi, s.vp.lo);
+      }
+      __syncwarp();  // before the next chunk overwrites the slots
     }
-    int sb = 0;
-    while (sb < ne) {
-      const int64_t pbeg = s_off[sb];
-      const bool fits = threadIdx.x >= sb && threadIdx.x < ne &&
-                        s_off[threadIdx.x + 1] - pbeg <= kNT &&
-                        s_poff[threadIdx.x + 1] - s_poff[sb] <= kPC;
-      const int sbe = sb + __syncthreads_count(fits);
-      if (sbe == sb) {  // one event larger than a sub-batch (particles or pairs)
-        if constexpr (FIX) big_event<LP, LS, LG>(A, T, e0 + sb, pbeg, s_off[sb + 1] - pbeg, s_poff[sb]);
-        else fix = true;
+  }
+  // (d)
+#pragma unroll 1
+  for (int r = 0; r < 2; r++) {
+    const int c = lane + 32 * r;
+    if (!(c < np && GVX_IN_BOUNDS(pb + c, A.n_particles, A.status))) break;
+    const int k = r ? rank[1] : rank[0];
+    const ffm::EvPart p = staged(W, c);
+    const float2 m = W.mm[c];
+    const uint32_t ew = W.scale[k] & 0x7ff00000u;
+    const V4<double> g64 = A.has_gsum ? ld4c<LS>(A.gsum, e0 + (W.info[k].w & 0xff)) : V4<double>{0.0, 0.0, 0.0, 0.0};
+    ffm::ff gs[4];
+    const uint32_t ewg = ffm::ev_gs(g64.x, g64.y, g64.z, g64.w, gs);
+    const bool fast = p.pt_hi >= 0.0f, done = !A.has_gsum || (fast && ewg != 1u);
+    if constexpr (!RARE) {
+      const ffm::EvOwn<ffm::ff> own = ffm::ev_own(p, ffm::ff{m.x, m.y});
+      const ffm::EvLeg<ffm::ff> l = ffm::ev_leg(own, T);
+      const float2 s0 = W.sum[0][c], s1 = W.sum[1][c], s2 = W.sum[2][c], s3 = W.sum[3][c], s4 = W.sum[4][c];
+      ffm::ff dpt, deta, dm;
+      ffm::ev_grad_terms(own, l, ffm::ff{s0.x, s0.y}, ffm::ff{s1.x, s1.y}, ffm::ff{s2.x, s2.y},
+                         ffm::ff{s3.x, s3.y}, &dpt, &deta, &dm);
+      V4<double> o = {ffm::ev_out(dpt, ffm::ev_off_pt()), ffm::ev_out(deta, ffm::ev_off_angle(ew)),
+                      ffm::ev_out(ffm::ff{s4.x, s4.y}, ffm::ev_off_angle(ew)), ffm::ev_out(dm, ffm::ev_off_pt())};
+      if (ewg > 1u) {
+        ffm::ff t[4];
+        ffm::ev_sum_terms(own, l, gs, T, t);
+        const uint32_t ep = ffm::ev_off_gs_pt(ewg), ea = ffm::ev_off_gs_angle(ewg, ew);
+        o = {o.x + ffm::ev_out(t[0], ep), o.y + ffm::ev_out(t[1], ea), o.z + ffm::ev_out(t[2], ea),
+             o.w + ffm::ev_out(t[3], ep)};
+      }
+      if (!fast) o = {0.0, 0.0, 0.0, 0.0};
+      rare |= !done;
+      st4<double, LG>(A.grad, pb + c, o);
+    } else {
+      V4<double> add = dg[c];
+      if (!done) {
+        const V4<double> sp = sum_part(ld4c<LP>(A.p, pb + c), g64);
+        add = {add.x + sp.x, add.y + sp.y, add.z + sp.z, add.w + sp.w};
+      }
+      if (add.x != 0.0 || add.y != 0.0 || add.z != 0.0 || add.w != 0.0) {
+        // plain coherent loads: the first launch wrote the array
+        const V4<double> was = ld4<double, LG>(
+            Lv{{A.grad.c[0], A.grad.c[1], A.grad.c[2], A.grad.c[3]}, A.grad.layout}, pb + c);
+        st4<double, LG>(A.grad, pb + c, V4<double>{was.x + add.x, was.y + add.y, was.z + add.z, was.w + add.w});
+      }
+    }
+  }
+  rare = __any_sync(kAll, rare);  // and the buffer may be overwritten
+  return rare;
+}
+
+// What one walk over a tile's batches shares among the warps.
+struct TileState {
+  int next;       // the next batch to take
+  unsigned rare;  // bit b: a batch of number b modulo 32 left something
+};
+
+// The tile's batches: in the first walk every warp takes one after another by number, in the second
+// the flagged ones are dealt out in turn.  *large: an event was left to the CTA.
+template <int LP, int LS, int LG, bool RARE>
+__device__ __forceinline__ void walk_tile(const BArgs &A, const ffm::LcTab &T, WarpBuf &W, TileState &S,
+                                          int64_t e0, int ne, const int64_t *s_off, const int64_t *s_po,
+                                          bool *large) {
+  const int lane = threadIdx.x & 31;
+  int mine = threadIdx.x >> 5, flagged = 0;
+  for (int sb = 0, number = 0; sb < ne;) {
+    const int64_t lo = s_off[min(sb + lane, ne)], hi = s_off[min(sb + lane + 1, ne)];
+    const int64_t pb = __shfl_sync(kAll, lo, 0);
+    int take = __popc(__ballot_sync(kAll, sb + lane < ne && hi - pb <= A.cap));
+    if (take == 0) {
+      if (__shfl_sync(kAll, hi, 0) - pb > kCapW) {
+        *large = true;
         sb++;
-        __syncthreads();
         continue;
       }
-      const int np = (int)(s_off[sbe] - pbeg);
-      const int ns = sbe - sb;
-      // (a) raw particles, the larger high word of pt and |m|; the events' order
-      if (k < np && GVX_IN_BOUNDS(pbeg + k, A.n_particles, A.status)) {
-        const V4<double> x = ld4c<LP>(A.p, pbeg + k);
-        s_pt[k] = x.x;
-        s_eta[k] = x.y;
-        s_phi[k] = x.z;
-        s_m[k] = x.w;
-        s_sc[k] = (int)ffm::umax32(ffm::dhi(x.x), ffm::dhi(x.w) & 0x7fffffffu);
-      }
-      if (threadIdx.x < ns) {  // rank of event sb + threadIdx.x: larger first, ties by position
-        const int me = sb + threadIdx.x;
-        const int64_t nme = s_off[me + 1] - s_off[me];
-        int rank = 0;
-        int64_t before = 0;  // particles of the events ranked ahead
-        for (int o = sb; o < sbe; o++) {
-          const int64_t no = s_off[o + 1] - s_off[o];
-          if (no > nme || (no == nme && o < me)) {
-            rank++;
-            before += no;
-          }
-        }
-        s_order[rank] = me;
-        s_start[rank] = (int)before;
-      }
-      __syncthreads();
-      // the particle this thread takes in (b) and (c): thread k holds position k of the sorted
-      // events
-      int e = 0, b0 = 0, li = 0, p = 0;
-      if (k < np) {
-        int r = 0, hi = ns - 1;
-        while (r < hi) {
-          const int mid = (r + hi + 1) >> 1;
-          if (s_start[mid] <= k) r = mid;
-          else hi = mid - 1;
-        }
-        e = s_order[r];
-        b0 = (int)(s_off[e] - pbeg);
-        li = k - s_start[r];
-        p = b0 + li;
-      }
-      const int n = k < np ? (int)(s_off[e + 1] - s_off[e]) : 0;
-      // (b) the particle's event scale, domain and light-cone terms
-      int sc = kNoFast;
-      if (k < np) {
-        uint32_t wmax = 0;
-        for (int t = b0; t < b0 + n; t++) wmax = ffm::umax32((uint32_t)s_sc[t], wmax);
-        const double pt = s_pt[p], eta = s_eta[p], phi = s_phi[p], m = s_m[p];
-        const uint32_t ew = wmax & 0x7ff00000u;
-        const uint32_t hp = ffm::dhi(pt), hm = ffm::dhi(m) & 0x7fffffffu;
-        const uint32_t he = ffm::dhi(eta) & 0x7fffffffu, hf = ffm::dhi(phi) & 0x7fffffffu;
-        if (wmax - (200u << 20) < (1700u << 20) &&
-            ffm::umin32(hp - 0x100000u, hm - 0x100000u) >= ew - (41u << 20) &&
-            ffm::umax32(hp, hm) >= 0x100000u && he < 0x40200000u && hf < 0x400C0000u) {
-          const uint32_t rb = ew - (127u << 20);
-          const ff pt_i = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(pt), rb));
-          const ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(m), rb));
-          const ff xe = ffm::cvt1(ffm::cvt_parts_normal(ffm::umax32(he, 0x3E100000u),
-                                                        ffm::dlo(eta), ffm::kRebaseOne));
-          ff sh, ch;
-          const ffm::LcLeg<ff> L = ffm::lc_leg(pt_i, mmf, xe, T.hyp, &sh, &ch);
-          s_pY[p] = pack4(pt_i, L.Y);
-          s_DE[p] = pack4(L.D, L.E);
-          s_cs[p] = pack4(ch, sh);
-          s_mm[p] = make_float2(mmf.hi, mmf.lo);
-          sc = (int)ew;
-        }
-        s_fs[p] = sc;
-        // the event-sum part starts the particle's FP64 slot
-        V4<double> sp = {0.0, 0.0, 0.0, 0.0};
-        if (A.has_gsum) {
-          const V4<double> gsv = ld4c<LS>(A.gsum, e0 + e);
-          const V4<double> xp = {pt, eta, phi, m};
-          bool done = false;
-          if (sc != kNoFast) {
-            const float4 pY = s_pY[p], DE = s_DE[p], cs = s_cs[p];
-            const float2 mm2 = s_mm[p];
-            done = sum_part_lc(ff{pY.x, pY.y}, ff{DE.z, DE.w}, ff{mm2.x, mm2.y}, ff{cs.x, cs.y},
-                               ff{cs.z, cs.w}, eta, phi, m, (uint32_t)sc - (127u << 20), gsv, T, &sp);
-          }
-          if constexpr (FIX) {  // only what the first launch left out
-            sp = done ? V4<double>{0.0, 0.0, 0.0, 0.0} : sum_part(xp, gsv);
-          } else if (!done) {
-            fix = true;
-          }
-        }
-        s_acc[p] = make_double4(sp.x, sp.y, sp.z, sp.w);
-      }
-      __syncthreads();
-      // (c) pair-parallel: each pair's angular terms, m and c = gm / (2m) once, into the pair's
-      // slot (the sd terms for the orientation (i, j), i < j); a pair outside the float-float
-      // domain gets the marker kSlowPair
-      const int64_t q0 = s_poff[sb];
-      const int npq = (int)(s_poff[sbe] - q0);
-      for (int q = threadIdx.x; q < npq; q += kNT) {
-        int lo = sb, hi = sbe - 1;  // the pair's event: the last with s_poff[ev] <= q0 + q
-        while (lo < hi) {
-          const int mid = (lo + hi + 1) >> 1;
-          if (s_poff[mid] <= q0 + q) lo = mid;
-          else hi = mid - 1;
-        }
-        int64_t i, j;
-        decode_pair(q0 + q - s_poff[lo], s_off[lo + 1] - s_off[lo], i, j);
-        const int ia = (int)(s_off[lo] - pbeg + i), ib = (int)(s_off[lo] - pbeg + j);
-        if (!(GVX_IN_BOUNDS(ia, np, A.status) && GVX_IN_BOUNDS(ib, np, A.status) &&
-              GVX_IN_BOUNDS(q, kPC, A.status) && GVX_IN_BOUNDS(q0 + q, A.n_pairs, A.status)))
-          continue;
-        const double g = __ldg(A.gpm + q0 + q);
-        const uint32_t hg = ffm::dhi(g) & 0x7fffffffu;
-        float4 w0 = make_float4(__uint_as_float(kSlowPair), 0.0f, 0.0f, 0.0f);
-        float4 w1 = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        if (s_fs[ia] != kNoFast && s_fs[ib] != kNoFast) {
-          if ((hg | ffm::dlo(g)) == 0u) {
-            w0 = w1;  // gm = 0: no contribution
-          } else if (hg - (963u << 20) < (81u << 20)) {  // |gm| in [2^-60, 2^20]
-            ff S;
-            ff2 sd;
-            const bool oka = ffm::lc_pair_angles(s_eta[ia], s_eta[ib], s_phi[ia], s_phi[ib], T, &S, &sd);
-            const float4 pa = s_pY[ia], pb = s_pY[ib], da = s_DE[ia], db = s_DE[ib];
-            ff m2s;
-            const bool okm = ffm::lc_pair_m2(ff{pa.x, pa.y}, ff{pb.x, pb.y}, ff{pa.z, pa.w},
-                                             ff{pb.z, pb.w}, ff{da.x, da.y}, ff{db.x, db.y}, S, &m2s);
-            if (oka && okm) {
-              w0 = w1;  // m = 0: the gradient is 0
-              if (m2s.hi != 0.0f) {
-                const ff m = ffm::lc_sqrt_refined(m2s);
-                const ff gf = ffm::cvt1(ffm::cvt_parts(hg, ffm::dlo(g), ffm::kRebaseOne));
-                const ff c = ffm::lc_scale(ffm::lc_div(gf, ff{ffm::fmul(m.hi, 2.0f), ffm::fmul(m.lo, 2.0f)}),
-                                           ffm::sign_of(g));
-                const ff cS = ffm::lc_mul(c, S);
-                const ff2 csd = ffm::lc_mul(ff2{ffm::bc2(c.hi), ffm::bc2(c.lo)}, sd);
-                w0 = make_float4(c.hi, c.lo, cS.hi, cS.lo);
-                w1 = make_float4(csd.hi.x, csd.lo.x, csd.hi.y, csd.lo.y);
-              }
-            }
-          }
-        }
-        s_w0[q] = w0;
-        s_w1[q] = w1;
-      }
-      __syncthreads();
-      // (d) per particle, its partners in order: seven float-float sums from the pair slots, the
-      // FP64 formulas for marked pairs; then the pair part and the conversion
-      if (k < np) {
-        const int slot0 = (int)(s_poff[e] - q0);  // the event's first pair slot
-        ff2 A12 = {ffm::bc2(0.0f), ffm::bc2(0.0f)};  // (A1, A2)
-        ff2 A34 = A12, A56 = A12;                    // (A3, A4), (A5, A6)
-        ff A7 = {0.0f, 0.0f};
-        // packed index of pair (min(li, j), max(li, j)): for j < li it is j n - j(j+1)/2 + li - j - 1
-        // (step n - j - 2), for j > li it is li n - li(li+1)/2 + j - li - 1 (step 1)
-        int idx = li - 1;  // the index for j = 0 (when li > 0)
-        for (int j = 0; j < n; j++) {
-          if (j == li) {
-            idx = li * n - li * (li + 1) / 2;  // the index for j = li + 1
-            continue;
-          }
-          const int pidx = idx;
-          idx += j < li ? n - j - 2 : 1;
-          const int q = b0 + j;
-          if (!(GVX_IN_BOUNDS(slot0 + pidx, npq, A.status) && GVX_IN_BOUNDS(q, np, A.status)))
-            continue;
-          const float4 w0 = s_w0[slot0 + pidx], w1 = s_w1[slot0 + pidx];
-          if constexpr (FIX) {  // the marked pairs only, into this thread's own slot
-            if (__float_as_uint(w0.x) == kSlowPair)
-              slow_pair_add(V4<double>{s_pt[p], s_eta[p], s_phi[p], s_m[p]},
-                            V4<double>{s_pt[q], s_eta[q], s_phi[q], s_m[q]},
-                            __ldg(A.gpm + s_poff[e] + pidx), s_acc + p);
-            continue;
-          }
-          if (__float_as_uint(w0.x) == kSlowPair) {  // left to the FIX launch
-            fix = true;
-            continue;
-          }
-          const float sg = j > li ? 1.0f : -1.0f;  // the slot's sd terms are for (min, max)
-          const float4 pY = s_pY[q], DE = s_DE[q];
-          const ff c = {w0.x, w0.y};
-          const ff2 cb = {ffm::bc2(c.hi), ffm::bc2(c.lo)};
-          A12 = ffm::add_same(A12, ffm::lc_mul(cb, ff2{ffm::mk2(DE.x, pY.z), ffm::mk2(DE.y, pY.w)}));
-          const ff cE = ffm::lc_mul(c, ff{DE.z, DE.w});
-          A34 = ffm::add_same(A34, ff2{ffm::mk2(c.hi, cE.hi), ffm::mk2(c.lo, cE.lo)});
-          const ff2 ptb = {ffm::bc2(pY.x), ffm::bc2(pY.y)};
-          A56 = ffm::add_same(A56, ffm::lc_mul(ptb, ff2{ffm::mk2(w0.z, sg * w1.x), ffm::mk2(w0.w, sg * w1.y)}));
-          A7 = ffm::add_same(A7, ffm::lc_mul(ff{pY.x, pY.y}, ff{sg * w1.z, sg * w1.w}));
-        }
-        // the pair part from the accumulators, plus the FP64 slot (event-sum part, slow pairs)
-        const double4 a = s_acc[p];
-        double out[4] = {a.x, a.y, a.z, a.w};
-        if constexpr (FIX) {
-          if (a.x != 0.0 || a.y != 0.0 || a.z != 0.0 || a.w != 0.0) {
-            // the first launch's value (plain coherent loads: this launch writes the array)
-            const V4<double> w = ld4<double, LG>(Lv{{A.grad.c[0], A.grad.c[1], A.grad.c[2], A.grad.c[3]},
-                                                    A.grad.layout}, pbeg + p);
-            st4<double, LG>(A.grad, pbeg + p, V4<double>{w.x + out[0], w.y + out[1], w.z + out[2], w.w + out[3]});
-          }
-        } else if (sc != kNoFast) {
-          const float4 DE = s_DE[p], cs = s_cs[p];
-          const float2 mm2 = s_mm[p];
-          const ff E_i = {DE.z, DE.w}, ch = {cs.x, cs.y}, sh = {cs.z, cs.w}, mm = {mm2.x, mm2.y};
-          const uint32_t eoff_s = (uint32_t)sc - (127u << 20);  // 2^s
-          const float4 pYi = s_pY[p];
-          const ff pt_i = {pYi.x, pYi.y}, Y_i = {pYi.z, pYi.w}, D_i = {DE.x, DE.y};
-          const ff2 yd = ffm::lc_mul(ff2{ffm::mk2(Y_i.hi, D_i.hi), ffm::mk2(Y_i.lo, D_i.lo)}, A12);
-          const ff G = ffm::add_same(ffm::lane_x(yd), ffm::lc_scale(ffm::lane_y(yd), -1.0f));  // Y A1 - D A2
-          const ff rE = ffm::lc_div(ff{1.0f, 0.0f}, E_i);
-          const float seta = ffm::sign_of(s_eta[p]), sm = ffm::sign_of(s_m[p]);
-          const ff dpt = ffm::add_same(ffm::lc_mul(ffm::lc_mul(ch, rE), G),
-                                       ff{ffm::fmul(ffm::lane_x(A56).hi, 4.0f), ffm::fmul(ffm::lane_x(A56).lo, 4.0f)});
-          const ff deta = ffm::add_same(ffm::lc_scale(ffm::lc_mul(ffm::lc_mul(ffm::lc_mul(pt_i, sh), rE), G), seta),
-                                        ffm::lc_mul(pt_i, ffm::lane_y(A56)));
-          const ff dphi = ffm::lc_mul(pt_i, A7);
-          const ff dm = ffm::lc_scale(ffm::lc_mul(ffm::lc_mul(mm, rE),
-                                                  ffm::add_same(ffm::lc_mul(E_i, ffm::lane_x(A34)), ffm::lane_y(A34))),
-                                      2.0f * sm);
-          constexpr uint32_t kUnscaled = 896u << 20;
-          out[0] += ffm::lc_to_double(dpt, kUnscaled);
-          out[1] += ffm::lc_to_double(deta, eoff_s);
-          out[2] += ffm::lc_to_double(dphi, eoff_s);
-          out[3] += ffm::lc_to_double(dm, kUnscaled);
-        }
-        if constexpr (!FIX) st4<double, LG>(A.grad, pbeg + p, V4<double>{out[0], out[1], out[2], out[3]});
-      }
-      __syncthreads();  // before the next sub-batch overwrites the staged particles
-      sb = sbe;
+      take = 1;
     }
-    if constexpr (!FIX) {  // list the tile for the FIX launch if any thread met an FP64 path
-      if (__syncthreads_or(fix) && threadIdx.x == 0) {
-        const unsigned long long q = atomicAdd(A.fix_count, 1ull);  // < n_tiles: one per tile
-        if (GVX_IN_BOUNDS(q, n_tiles, A.status)) A.fix_tiles[q] = tile;
-      }
-      fix = false;
+    bool here;
+    if constexpr (RARE) {
+      const bool f = (S.rare >> (number & 31)) & 1u;
+      here = f && (flagged & (kNT / 32 - 1)) == mine;
+      flagged += f;
+    } else {
+      here = number == mine;
     }
+    if (here) {
+      const bool rare = warp_batch<LP, LS, LG, RARE>(A, T, W, e0, sb, take, lo, hi, s_po);
+      if constexpr (!RARE) {
+        int t = 0;
+        if (lane == 0) {
+          if (rare) atomicOr(&S.rare, 1u << (number & 31));
+          t = atomicAdd(&S.next, 1);
+        }
+        mine = __shfl_sync(kAll, t, 0);
+      }
+    }
+    number++;
+    sb += take;
   }
 }
 
-template <int LP, int LS, int LG, bool FIX>
-cudaError_t launch_one(const BArgs &A, cudaStream_t s) {
-  constexpr auto k = event_pairs_bwd_kernel<LP, LS, LG, FIX>;
-  cudaError_t err =
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
-  if (err != cudaSuccess) return err;
-  const int64_t n_tiles = (A.n_events + kTE - 1) / kTE;
-  const unsigned grid = balanced_grid_of<k>(kNT, kDynSmem, n_tiles, 1);  // one tile per CTA and pass
-  k<<<grid, kNT, kDynSmem, s>>>(A);
-  return cudaGetLastError();
+constexpr unsigned long long kLarge = 1ull << 32;
+
+// A tile's offsets into shared memory; false for a tile whose offsets cannot be right.
+__device__ __forceinline__ bool load_tile(const BArgs &A, int64_t e0, int ne, int64_t *s_off, int64_t *s_po) {
+  for (int k = threadIdx.x; k <= ne; k += kNT) {
+    s_off[k] = A.off[e0 + k];
+    s_po[k] = A.pair_off[e0 + k];
+  }
+  __syncthreads();
+  bool bad = false;
+  if (threadIdx.x < ne) {
+    const int64_t a = s_off[threadIdx.x], b = s_off[threadIdx.x + 1], n = b - a;
+    const int64_t pa = s_po[threadIdx.x], pb = s_po[threadIdx.x + 1];
+    bad = a < 0 || n < 0 || b > A.n_particles || n > (1ll << 31) || pa < 0 || pb > A.n_pairs ||
+          pb - pa != n * (n - 1) / 2;
+    if (e0 + threadIdx.x == 0 && (a != 0 || pa != 0)) bad = true;
+  }
+  return !__syncthreads_or(bad);
 }
 
-// The list count zeroed, the staged launch, then the FIX launch (which has nothing to do unless
-// the first listed tiles).
 template <int LP, int LS, int LG>
-cudaError_t launch_l(const BArgs &A, cudaStream_t s) {
-  cudaError_t err = cudaMemsetAsync(A.fix_count, 0, sizeof(unsigned long long), s);
+__global__ void __launch_bounds__(kNT, kCtas) event_pairs_bwd_kernel(const __grid_constant__ BArgs A) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  WarpBuf *bufs = reinterpret_cast<WarpBuf *>(s_dyn);
+  __shared__ int64_t s_off[kTE + 1], s_po[kTE + 1];
+  __shared__ TileState s_tile;
+  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
+  const int64_t n_tiles = (A.n_events + A.te - 1) / A.te;
+  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    const int64_t e0 = tile * A.te;
+    const int ne = (int)(A.n_events - e0 < A.te ? A.n_events - e0 : A.te);
+    __syncthreads();  // the previous tile is done with the shared arrays
+    if (threadIdx.x == 0) s_tile = {kNT / 32, 0u};
+    unsigned long long left = 0;
+    if (load_tile(A, e0, ne, s_off, s_po)) {
+      bool large = false;
+      walk_tile<LP, LS, LG, false>(A, T, bufs[threadIdx.x >> 5], s_tile, e0, ne, s_off, s_po, &large);
+      __syncthreads();
+      left = s_tile.rare | (large ? kLarge : 0ull);
+    } else if (threadIdx.x == 0) {
+      raise_status(A.status, GVX_ERR_OFFSETS);
+    }
+    if (threadIdx.x == 0) A.left[tile] = left;
+  }
+}
+
+// What the first launch left (nothing, most of the time): every block scans its part of the tiles'
+// words and takes the tiles that have one.  A launch of its own, because a call anywhere in the first
+// kernel costs its batches spills (413 us against 392 us at 300,007 events).
+template <int LP, int LS, int LG>
+__global__ void __launch_bounds__(kNT, 4) event_pairs_bwd_left_kernel(const __grid_constant__ BArgs A) {
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  WarpBuf *bufs = reinterpret_cast<WarpBuf *>(s_dyn);
+  __shared__ int64_t s_off[kTE + 1], s_po[kTE + 1];
+  __shared__ TileState s_tile;
+  __shared__ unsigned long long s_left[kNT];
+  const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
+  const int64_t n_tiles = (A.n_events + A.te - 1) / A.te;
+  // the block's tiles: every gridDim.x-th, a thread looking at one (so that neighbouring tiles, often
+  // alike, go to different blocks)
+  for (int64_t t0 = blockIdx.x; t0 < n_tiles; t0 += (int64_t)gridDim.x * kNT) {
+    const int64_t t = t0 + (int64_t)gridDim.x * threadIdx.x;
+    const unsigned long long mine = t < n_tiles ? A.left[t] : 0ull;
+    if (!__syncthreads_or(mine != 0ull)) continue;
+    s_left[threadIdx.x] = mine;
+    __syncthreads();
+    for (int k = 0; k < kNT; k++) {
+      const unsigned long long left = s_left[k];
+      if (left == 0ull) continue;
+      const int64_t e0 = (t0 + (int64_t)gridDim.x * k) * A.te;
+      const int ne = (int)(A.n_events - e0 < A.te ? A.n_events - e0 : A.te);
+      __syncthreads();  // the previous tile is done with the shared arrays
+      if (threadIdx.x == 0) s_tile = {0, (unsigned)left};
+      if (!load_tile(A, e0, ne, s_off, s_po)) continue;
+      bool large;
+      if ((unsigned)left != 0u)
+        walk_tile<LP, LS, LG, true>(A, T, bufs[threadIdx.x >> 5], s_tile, e0, ne, s_off, s_po, &large);
+      if (left & kLarge)
+        for (int e = 0; e < ne; e++)
+          if (s_off[e + 1] - s_off[e] > kCapW)
+            big_event<LP, LS, LG>(A, T, e0 + e, s_off[e], s_off[e + 1] - s_off[e], s_po[e]);
+    }
+    __syncthreads();
+  }
+}
+
+// Events per tile and particles per batch: whole tiles of kTE where they make kTileWaves per CTA that
+// fits at once, smaller ones below (100,000 events: 143 us at 4 waves, 147 at 2, 167 at 1), and at the
+// last step smaller batches, so that more warps share them (20,000 events: 46 us, with whole batches 48).
+constexpr int kTileWaves = 4;
+void tile_shape(int64_t n_events, int *te, int *cap) {
+  const int64_t ctas = (int64_t)num_sms() * kCtas * kTileWaves;
+  *te = kTE;
+  *cap = kCapW;
+  while (*te > kMinTE && n_events < *te * ctas) *te /= 2;
+  if (*te == kMinTE) *cap = 32;
+}
+
+template <int LP, int LS, int LG>
+cudaError_t launch_l(BArgs A, cudaStream_t s) {
+  constexpr auto k = event_pairs_bwd_kernel<LP, LS, LG>, left = event_pairs_bwd_left_kernel<LP, LS, LG>;
+  cudaError_t err =
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
+  if (err == cudaSuccess)
+    err = cudaFuncSetAttribute(left, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDynSmem);
   if (err != cudaSuccess) return err;
-  err = launch_one<LP, LS, LG, false>(A, s);
+  tile_shape(A.n_events, &A.te, &A.cap);
+  const int64_t n_tiles = (A.n_events + A.te - 1) / A.te;
+  k<<<balanced_grid_of<k>(kNT, kDynSmem, n_tiles, 1), kNT, kDynSmem, s>>>(A);  // one tile per CTA and pass
+  err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  return launch_one<LP, LS, LG, true>(A, s);
+  left<<<balanced_grid_of<left>(kNT, kDynSmem, n_tiles, 1, 1), kNT, kDynSmem, s>>>(A);
+  return cudaGetLastError();
 }
 
 }  // namespace
 
 size_t event_pairs_bwd_workspace(int64_t n_events) {
-  return kWsList + (size_t)((n_events + kTE - 1) / kTE) * sizeof(int64_t);
+  return 256 + (size_t)((n_events + kWsEvents - 1) / kWsEvents) * sizeof(unsigned long long);
 }
 
 cudaError_t launch_event_pairs_bwd(const Lv &p, const int64_t *off, const int64_t *pair_off,
@@ -564,8 +628,7 @@ cudaError_t launch_event_pairs_bwd(const Lv &p, const int64_t *off, const int64_
   A.gsum = gsum ? *gsum : Lv{{nullptr, nullptr, nullptr, nullptr}, GVX_SOA};
   A.grad = grad;
   A.status = device_status_word();
-  A.fix_count = (unsigned long long *)ws;
-  A.fix_tiles = (int64_t *)((char *)ws + kWsList);
+  A.left = (unsigned long long *)ws;
   const int lp = p.layout, ls = A.gsum.layout, lg = grad.layout;
   if (lp == GVX_SOA) {
     if (ls == GVX_SOA) return lg == GVX_SOA ? launch_l<GVX_SOA, GVX_SOA, GVX_SOA>(A, s)
