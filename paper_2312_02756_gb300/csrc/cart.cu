@@ -361,18 +361,19 @@ cudaError_t launch_ptetaphie_t(const Lv &a, const Lv &b, T *m, int64_t n, cudaSt
     }
     return cudaGetLastError();
   }
+  constexpr int threads64 = 128;  // in 32 waves, as the Cartesian masses: 156 -> 149 us at 10,000,019 pairs
   if (a.layout == GVX_SOA && b.layout == GVX_SOA) {
     constexpr auto k = mass_ptetaphie_kernel<T, GVX_SOA, GVX_SOA>;
-    k<<<balanced_grid_of<k>(threads, 0, n), threads, 0, s>>>(a, b, m, n);
+    k<<<balanced_grid_of<k>(threads64, 0, n, 0, 32), threads64, 0, s>>>(a, b, m, n);
   } else if (a.layout == GVX_SOA) {
     constexpr auto k = mass_ptetaphie_kernel<T, GVX_SOA, GVX_AOS>;
-    k<<<balanced_grid_of<k>(threads, 0, n), threads, 0, s>>>(a, b, m, n);
+    k<<<balanced_grid_of<k>(threads64, 0, n, 0, 32), threads64, 0, s>>>(a, b, m, n);
   } else if (b.layout == GVX_SOA) {
     constexpr auto k = mass_ptetaphie_kernel<T, GVX_AOS, GVX_SOA>;
-    k<<<balanced_grid_of<k>(threads, 0, n), threads, 0, s>>>(a, b, m, n);
+    k<<<balanced_grid_of<k>(threads64, 0, n, 0, 32), threads64, 0, s>>>(a, b, m, n);
   } else {
     constexpr auto k = mass_ptetaphie_kernel<T, GVX_AOS, GVX_AOS>;
-    k<<<balanced_grid_of<k>(threads, 0, n), threads, 0, s>>>(a, b, m, n);
+    k<<<balanced_grid_of<k>(threads64, 0, n, 0, 32), threads64, 0, s>>>(a, b, m, n);
   }
   return cudaGetLastError();
 }
