@@ -13,9 +13,10 @@
 // taken in float-float, and scaled back: the relative error of m is below 2^-44.  Integer and FP32
 // pipes only, plus one FP64 add for the final rounding (none for FP32 output).
 //
-// Bound by issue with the loads (10,000,019 FP64 pairs as rows: 153 us, 4.7 TB/s of the 72 bytes a pair,
-// 406 warp instructions per 32 pairs).  Three 32-bit words per magnitude, with compares for the signs of
-// the sums and carries through every product, took 188 us and 511 instructions.
+// Bound by issue with the loads (10,000,019 FP64 pairs as rows: 143 us, 5.0 TB/s of the 72 bytes a pair,
+// 420 warp instructions per 32 pairs).  In the same launch shape (256 threads) it took 153 us, and three
+// 32-bit words per magnitude, with compares for the signs of the sums and carries through every product,
+// 188 us and 511 instructions.
 //
 // Outside the fast path (a non-finite component, a scale exponent outside [-900, 900] for double
 // or [-100, 100] for float input, or |m^2| below the threshold, zero included) the functions

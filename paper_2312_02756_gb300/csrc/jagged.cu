@@ -24,7 +24,7 @@
 //      staged the same way up to kCP particles, straight from global memory beyond.
 // Tile descriptors are 64-bit words: 2 flag bits (aggregate / inclusive prefix) + 62-bit value.
 //
-// Bound by issue and the shared-memory/L1 data pipe together (430 warp instructions and 115 data
+// Bound by issue and the shared-memory/L1 data pipe together (440 warp instructions and 104 data
 // wavefronts per 32 pairs, of which the two table gathers take about 40).  2^20 events, 33.5 M
 // pairs: 0.558 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
 // and a search per pair (620 instructions per 32 pairs, FP64 pipe 35% busy).  Six CTAs of 128
