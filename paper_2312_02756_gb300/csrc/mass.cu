@@ -31,6 +31,12 @@ constexpr int kUnroll = 4;
 // SMs' progress).
 constexpr int kMassWaves = 32;
 
+// Forward, from two waves of it on: fewer waves where 32 would leave a thread less than this many pairs,
+// because a CTA's first loads have no prefetch before them.  Columns, 3,000,000 pairs: 62.8 us with 32
+// waves, 57.4 us so; 2^22 83.0 and 77.5; 2^24 276 and 269.5; equal from 2^25 on.  Below two waves the
+// steps are uneven: 2^20 pairs 28.7 us with 32 waves, 29.8 us so.
+constexpr int kMassSteps = 6;
+
 template <typename T, int LA, int LB>
 __global__ void __launch_bounds__(256) mass_kernel(Lv a, Lv b, T *__restrict__ m, int64_t n) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -185,9 +191,12 @@ __global__ void __launch_bounds__(256) mass_bwd_kernel(Lv a, Lv b, const T *__re
 
 template <int LA, int LB>
 void launch_mass_f64_l(const Lv &a, const Lv &b, double *m, int64_t n, cudaStream_t s) {
+  constexpr auto k = mass_f64_kernel<LA, LB>;
   const int threads = 128;
-  mass_f64_kernel<LA, LB><<<balanced_grid_of<mass_f64_kernel<LA, LB>>(threads, 0, n, 0, kMassWaves),
-                            threads, 0, s>>>(a, b, m, n);
+  const unsigned wave = balanced_grid_of<k>(threads, 0, n, 0, 1);
+  unsigned grid = balanced_grid_of<k>(threads, 0, n, threads * kMassSteps, kMassWaves);
+  if (grid < 2 * wave) grid = balanced_grid_of<k>(threads, 0, n, 0, kMassWaves);
+  k<<<grid, threads, 0, s>>>(a, b, m, n);
 }
 
 cudaError_t launch_mass_f64(const Lv &a, const Lv &b, void *m, int64_t n, cudaStream_t s) {
