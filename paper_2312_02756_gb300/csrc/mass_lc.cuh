@@ -377,13 +377,6 @@ GVX_HD void sincos_lc_at(const ff &r, uint32_t n, const gvx_f4 *sintab, ff *sn, 
   *sn = tab_comb_any(Sj, Cj, r, tp);
   *cs = tab_comb_any(Cj, ff{-Sj.hi, -Sj.lo}, r, tp);
 }
-// The same from x itself (x.lo in [0, ulp(x.hi))).
-GVX_HD void sincos_lc(const ff &x, const gvx_f4 *sintab, ff *sn, ff *cs) {
-  uint32_t j[1];
-  const ff r = lc_reduce(x, j);
-  sincos_lc_at(r, j[0], sintab, sn, cs);
-}
-
 // ---- the pair ------------------------------------------------------------------------------
 
 // The angular factor of a pair, S = sinh^2(|d_eta|/2) + sin^2(|d_phi|/2), from its raw angles,
