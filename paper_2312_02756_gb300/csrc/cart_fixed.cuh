@@ -81,8 +81,10 @@ struct Fmt<float> {
 GVX_HD uint32_t top_word(double x) { return ffm::dhi(x); }
 GVX_HD uint32_t top_word(float x) { return ffm::f2u(x); }
 
-// The significand with its leading bit at bit 63, as two words (a zero or denormal as if its
-// exponent were normal; the callers clear it).
+// The significand with its leading bit at bit 63, as two words.  A zero or denormal counts as 0 (it
+// lies below the units of every scale but the lowest FP32 ones): a float's significand is cleared here,
+// because at scale exponent -100 its exponent field of 0 is only 27 binades down; a double's, at least
+// 123 binades down, is shifted out of the outer limbs by limbs_near, which masks the middle one.
 struct Sig {
   uint32_t hi, lo;
 };
@@ -90,7 +92,7 @@ GVX_HD Sig significand(double x, uint32_t wh) {
   const uint32_t h = (wh & 0xfffffu) | 0x100000u, l = ffm::dlo(x);
   return {(h << 11) | (l >> 21), l << 11};
 }
-GVX_HD Sig significand(float, uint32_t w) { return {(w << 8) | 0x80000000u, 0u}; }
+GVX_HD Sig significand(float, uint32_t w) { return {(w & 0x7f800000u) ? (w << 8) | 0x80000000u : 0u, 0u}; }
 
 // A value of the scaled fixed point, in limbs of kLimb bits (those of a sum of two may be
 // negative or one bit longer).
