@@ -19,8 +19,9 @@
 // 188 us and 511 instructions.
 //
 // Outside the fast path (a non-finite component, a scale exponent outside [-900, 900] for double
-// or [-100, 100] for float input, or |m^2| below the threshold, zero included) the functions
-// return false and the caller evaluates the cancellation-free FP64 form.
+// or [-100, 100] for float input, a denormal float at a scale exponent below -43, or |m^2| below the
+// threshold, zero included) the functions return false and the caller evaluates the cancellation-free
+// FP64 form.
 #pragma once
 
 #include "ff.cuh"
@@ -82,9 +83,10 @@ GVX_HD uint32_t top_word(double x) { return ffm::dhi(x); }
 GVX_HD uint32_t top_word(float x) { return ffm::f2u(x); }
 
 // The significand with its leading bit at bit 63, as two words.  A zero or denormal counts as 0 (it
-// lies below the units of every scale but the lowest FP32 ones): a float's significand is cleared here,
-// because at scale exponent -100 its exponent field of 0 is only 27 binades down; a double's, at least
-// 123 binades down, is shifted out of the outer limbs by limbs_near, which masks the middle one.
+// lies below the units; m2_fixed declines the lowest FP32 scales, where a denormal does not): a float's
+// significand is cleared here, because at scale exponent -100 its exponent field of 0 is only 27
+// binades down; a double's, at least 123 binades down, is shifted out of the outer limbs by limbs_near,
+// which masks the middle one.
 struct Sig {
   uint32_t hi, lo;
 };
@@ -130,6 +132,13 @@ GVX_HD bool m2_fixed(const T *a, const T *b, i128 *m2, int *sc) {
   }
   const int emax = (int)(wmax >> kB), s = emax - Fmt<T>::kBias;
   if (emax == Fmt<T>::kMaxE || s < -Fmt<T>::kScaleLim || s > Fmt<T>::kScaleLim) return false;
+  if constexpr (sizeof(T) == 4) {  // a denormal component (below 2^-126) above the units of the scale
+    if (s < kFrac - 126) {
+#pragma unroll
+      for (int k = 0; k < 8; k++)
+        if ((w[k] & 0x7fffffffu) - 1u < 0x7fffffu) return false;
+    }
+  }
   const bool far = (uint32_t)emax - ((wmin + (1u << kB)) >> kB) > 20u;
   // the sums of the components, limb by limb and without carries
   Limbs S[4];

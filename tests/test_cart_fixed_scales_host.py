@@ -26,9 +26,9 @@ def _legs(s, dtype, n):
     return tuple(np.where(np.abs(v) < np.finfo(dtype).tiny, 0.0, v) for v in (a, b))
 
 
-def _check(got, ok, ref, tol):
+def _check(got, ok, ref, tol, least=0.5):
     hit = ok & (ref != 0.0)
-    assert hit.mean() > 0.5
+    assert hit.mean() > least
     assert np.max(np.abs(got - ref)[hit] / np.abs(ref[hit])) <= tol
 
 
@@ -46,3 +46,17 @@ def test_f64_scales(ffh, orc, s):  # noqa: F811
     for x, y in ((a, b), (b, a)):
         m, ok, _, _ = _cart_fixed(ffh, x, y)
         _check(m, ok, orc.mass_cart_def(x, y, "pxpypze"), 2.0 ** -44)
+
+
+@pytest.mark.parametrize("s", [-100, -97, -80, -60, -44, -43, -42])
+def test_f32_denormal_components(ffh, orc, s):  # noqa: F811
+    """A denormal component counts like any other: a pair with one is right, or declined where it would
+    lie above the units (2^-83 of the scale)."""
+    g = syn.rng(553)
+    a, b = _legs(s, np.float32, 8000)
+    for v in (a, b):
+        low = g.random(v.shape) < 0.15
+        low[:, 3] = False
+        v[low] = (g.integers(1, 1 << 23, low.sum()) * g.choice([-1.0, 1.0], low.sum())) * 2.0 ** -149
+    _, _, m, ok = _cart_fixed(ffh, a, b)
+    _check(m.astype(np.float64), ok, orc.mass_cart_def(a, b, "pxpypze"), 2.0 ** -24 * 1.01, 0.2)
