@@ -305,7 +305,8 @@ __device__ __forceinline__ int warp_batch(const JArgs &A, const ffm::LcTab &T, W
       extreme |= !stage_particle<RARE>(S, c, x[r], W.scale[rank[r]], T);
     }
   }
-  extreme = __any_sync(kAll, extreme);  // and the staged places are visible to the warp
+  extreme = __any_sync(kAll, extreme);
+  __syncwarp();  // the staged places and rows are visible to the warp (a vote orders no memory)
   // event sums: lanes (event, component pair, every other particle); an event with a particle
   // outside the float-float domain gets its sums in the second walk
   if (!RARE || extreme) {

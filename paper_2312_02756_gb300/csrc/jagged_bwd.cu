@@ -301,7 +301,8 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
       for (int k = 0; k < 5; k++) W.sum[k][c] = make_float2(0.0f, 0.0f);
     }
   }
-  const bool extreme = __any_sync(kAll, rare);  // and the staged places are visible to the warp
+  const bool extreme = __any_sync(kAll, rare);
+  __syncwarp();  // the staged places and rows are visible to the warp (a vote orders no memory)
   int rows = -1;  // rows that start before the current word, less one
   for (int c0 = 0; c0 < total; c0 += kPC) {
     const int c1 = c0 + kPC < total ? c0 + kPC : total;
@@ -437,7 +438,8 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
       }
     }
   }
-  rare = __any_sync(kAll, rare);  // and the buffer may be overwritten
+  rare = __any_sync(kAll, rare);
+  __syncwarp();  // the buffer may be overwritten
   return rare;
 }
 

@@ -292,6 +292,7 @@ __device__ __forceinline__ void offer(WarpBuf &W, bool valid, int e, double m, i
   if (valid) atomicMin(&W.key[e], key);
   __syncwarp();
   bool cand = valid && key == W.key[e];
+  __syncwarp();  // every lane has read its key before the next round lowers one
   while (__any_sync(kAll, cand)) {
     if (cand) W.own[e] = lane;
     __syncwarp();
@@ -415,7 +416,8 @@ __device__ __forceinline__ int warp_tile(const SArgs &A, const ffm::LcTab &T, Wa
           bool extreme = false;
           for (int c = lane; c < ns; c += 32)
             extreme |= !stage_leg(W.part[c], W.scale[W.part[c].tag >> 8], T);
-          extreme = __any_sync(kAll, extreme);  // and the staged places are visible to the warp
+          extreme = __any_sync(kAll, extreme);
+          __syncwarp();  // the staged places are visible to the warp (a vote orders no memory)
           bool rare = false;
           for (int r0 = 0; r0 < total; r0 += 32) {
             const int q = r0 + lane;
