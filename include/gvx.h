@@ -208,7 +208,9 @@ size_t gvx_event_pair_masses_workspace(int64_t n_events);
  *                  event's pairs in row-major order k(i,j) = i n - i(i+1)/2 + (j - i - 1).
  *   pair_capacity: length of pair_m; if the total is larger, nothing beyond it is written and
  *                  GVX_ERR_CAPACITY is recorded in the device status word.
- *   event_sum:     out, n_events PxPyPzE vectors (SoA or AoS): the sum of each event's particles.
+ *   event_sum:     out, n_events PxPyPzE vectors (SoA or AoS): the sum of each event's particles,
+ *                  each particle's components within 1e-12 of its energy, and for small angles py
+ *                  within 1e-12 of itself (phi near 0) and pz likewise (eta near 0).
  *   workspace:     gvx_event_pair_masses_workspace(n_events) bytes of device memory.
  * Events with more than 64 particles are supported (processed by a slower branch).  Malformed
  * offsets are detected on the device and recorded as GVX_ERR_OFFSETS.  One launch.

@@ -5,7 +5,7 @@
 // angle difference is then one exact integer subtraction, and its reduction to the table step
 // (h = d/2 = n 2^-8 + r) is bit fields of it.  An FP64 subtraction instead holds the FP64 pipe for
 // ~77 cycles per warp and is followed by a conversion of the difference by its bits; the integer
-// route issues about as many instructions and leaves that pipe idle.  A difference carries at most
+// route issues about as many instructions and leaves that pipe idle.  A difference carries about
 // 2^-59 of rounding from its two angles, so S = sinh^2(d_eta/2) + sin^2(d_phi/2) keeps 2^-47
 // relative where it is at least 2^-22 (kFxMinS); nearer pairs go to the elementwise arithmetic,
 // which subtracts the angles in FP64.
@@ -18,14 +18,16 @@ namespace ffm {
 
 constexpr float kFxMinS = 2.384185791015625e-07f;  // 2^-22
 
-// x, |x| < 8, in units of 2^-59, rounded to nearest (ties away from zero).
+// x, |x| < 8, in units of 2^-59, rounded to nearest (ties away from zero), a nonzero x to at least one
+// unit: 0 stands for 0 alone, and the sign is kept.
 GVX_HD int64_t angle_fx(double x) {
   const uint32_t wh = dhi(x), wl = dlo(x);
   // the significand with one guard bit, at the place it has for x in [4, 8)
   const uint64_t M = (((uint64_t)((wh & 0xfffffu) | 0x100000u) << 32) | wl) << 10;
   const uint32_t sh = 1025u - ((wh >> 20) & 0x7ffu);
   const uint64_t v = sh < 64u ? M >> sh : 0;
-  const int64_t r = (int64_t)((v + 1) >> 1);
+  int64_t r = (int64_t)((v + 1) >> 1);
+  if (r == 0 && ((wh << 1) | wl) != 0u) r = 1;
   return (wh >> 31) ? -r : r;
 }
 
@@ -49,6 +51,19 @@ GVX_HD ff fx_half_reduce(int64_t d, uint32_t *n) {
   // 2^-39 and 2^-60, negated for a negative difference
   const uint32_t sg = (uint32_t)dh & 0x80000000u;
   return {fmul(hi, u2f((88u << 23) | sg)), fmul(lo, u2f((67u << 23) | sg))};
+}
+
+// Whether an angle or a difference of two (units 2^-59) is nearer than 2^-12 to 0, where the rounding
+// to units is more than 2^-48 of it.
+GVX_HD bool fx_small(int64_t d) { return (uint32_t)((int32_t)(d >> 32) + (1 << 15)) < (1u << 16); }
+
+// |x| = n 2^-8 + r of a particle's own angle x, staged as a: fx_half_reduce of 2 a, for a small angle
+// r from x itself.  sinh(eta) and sin(phi) are factors of the particle's components, which keep
+// their relative accuracy however small the angle.
+GVX_HD ff own_reduce(double x, int64_t a, uint32_t *n) {
+  ff r = fx_half_reduce(2 * a, n);
+  if (fx_small(a)) r = cvt1(cvt_parts(dhi(x) & 0x7fffffffu, dlo(x), kRebaseOne));  // n is 0
+  return r;
 }
 
 // d_phi modulo 2 pi into about [-pi, pi] (2 pi to 2^-60: the difference stays good to 2^-59 where

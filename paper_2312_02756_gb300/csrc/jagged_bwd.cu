@@ -406,7 +406,12 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
     const uint32_t ewg = ffm::ev_gs(g64.x, g64.y, g64.z, g64.w, gs);
     const bool fast = p.pt_hi >= 0.0f, done = !A.has_gsum || (fast && ewg != 1u);
     if constexpr (!RARE) {
-      const ffm::EvOwn<ffm::ff> own = ffm::ev_own(p, ffm::ff{m.x, m.y});
+      ffm::EvOwn<ffm::ff> own = ffm::ev_own(p, ffm::ff{m.x, m.y});
+      if (ffm::fx_small(p.eta) || ffm::fx_small(p.phi)) {  // the angles themselves, seldom
+        const V4<double> v = ld4c<LP>(A.p, pb + c);
+        own.re = ffm::own_reduce(v.y, p.eta, &own.n[0]);
+        own.rp = ffm::own_reduce(v.z, p.phi, &own.j[0]);
+      }
       const ffm::EvLeg<ffm::ff> l = ffm::ev_leg(own, T);
       const float2 s0 = W.sum[0][c], s1 = W.sum[1][c], s2 = W.sum[2][c], s3 = W.sum[3][c], s4 = W.sum[4][c];
       ffm::ff dpt, deta, dm;
