@@ -55,7 +55,9 @@ GVX_HD ff fx_half_reduce(int64_t d, uint32_t *n) {
 
 // Whether an angle or a difference of two (units 2^-59) is nearer than 2^-12 to 0, where the rounding
 // to units is more than 2^-48 of it.
-GVX_HD bool fx_small(int64_t d) { return (uint32_t)((int32_t)(d >> 32) + (1 << 15)) < (1u << 16); }
+GVX_HD uint32_t fx_near0(int64_t d) { return (uint32_t)((int32_t)(d >> 32) + (1 << 15)); }
+GVX_HD bool fx_small(int64_t d) { return fx_near0(d) < (1u << 16); }
+GVX_HD bool fx_small(int64_t d, int64_t e) { return umin32(fx_near0(d), fx_near0(e)) < (1u << 16); }  // either
 
 // |x| = n 2^-8 + r of a particle's own angle x, staged as a: fx_half_reduce of 2 a, for a small angle
 // r from x itself.  sinh(eta) and sin(phi) are factors of the particle's components, which keep
@@ -125,12 +127,9 @@ GVX_HD bool ev_pair_m2(const EvPart &a, const EvPart &b, const LcTab &T, ff *m2s
 // Whether a staged angle is the FP64 one exactly: its last bit is at least 2^-59 from 2^-7 on.
 GVX_HD bool fx_exact(int64_t a) { return (a < 0 ? -a : a) >= (1ll << 52) || a == 0; }
 
-// Whether a pair's angle differences are exact (no angle below 2^-7, no turn taken off d_phi): then
-// S is good below kFxMinS too, and a launch seldom leaves a pair (one near pair in a hundred).
-GVX_HD bool ev_near_exact(const EvPart &a, const EvPart &b) {
-  const int64_t dp = a.phi - b.phi;
-  return fx_exact(a.eta) && fx_exact(b.eta) && fx_exact(a.phi) && fx_exact(b.phi) && wrap_fx(dp) == dp;
-}
+
+// Whether both angles of a staged particle are exact.
+GVX_HD bool ev_exact(int64_t eta, int64_t phi) { return fx_exact(eta) && fx_exact(phi); }
 
 }  // namespace ffm
 }  // namespace gvx

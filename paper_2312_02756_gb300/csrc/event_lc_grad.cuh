@@ -27,27 +27,48 @@ struct EvGrad {
   ff vp;
 };
 
+// |d|/2 of a small difference as ff (the table step is 0).
+GVX_HD ff small_half(double d) { return cvt1(cvt_parts(dhi(d) & 0x7fffffffu, dlo(d), kRebaseHalf)); }
+
 // The angular terms from staged angles: S = sinh^2(d_eta/2) + sin^2(d_phi/2) and
-// sd = (2 sinh d_eta, 2 sin d_phi).  False where S is below kFxMinS.
-GVX_HD bool lc_pair_angles_fx(int64_t eta1, int64_t phi1, int64_t eta2, int64_t phi2, const LcTab &T,
-                              ff *S, ff2 *sd) {
+// sd = (2 sinh d_eta, 2 sin d_phi), each of which enters a component of the gradient by itself, so that
+// either difference has to be good relatively.  It is where it is at least 2^-12 (to 2^-47) or between
+// exact angles (exact: all four are); of the others, about one pair in 10^6, near(d) gives the FP64
+// differences d[0], d[1] of the angles themselves.  False where it cannot, or where S is below kFxMinS
+// after a turn taken off d_phi.  (A turned d_phi is good to 2^-60, better than the FP64 difference.)
+template <class Near>
+GVX_HD bool lc_pair_angles_fx(int64_t eta1, int64_t phi1, int64_t eta2, int64_t phi2, bool exact, const Near &near,
+                              const LcTab &T, ff *S, ff2 *sd) {
   uint32_t n, j;
-  const int64_t de = eta1 - eta2, dp = wrap_fx(phi1 - phi2);
-  const ff re = fx_half_reduce(de, &n), rp = fx_half_reduce(dp, &j);
+  const int64_t de = eta1 - eta2, raw = phi1 - phi2, dp = wrap_fx(raw);
+  ff re = fx_half_reduce(de, &n), rp = fx_half_reduce(dp, &j);
+  uint32_t se = (uint32_t)(de >> 32), sp = (uint32_t)(dp >> 32);
+  bool good = true;
+  if (!exact && fx_small(de, dp)) {
+    double d[2] = {0.0, 0.0};
+    good = near(d);
+    if (fx_small(de)) {
+      re = small_half(d[0]);
+      se = dhi(d[0]);
+    }
+    if (fx_small(dp) && dp == raw) {
+      rp = small_half(d[1]);
+      sp = dhi(d[1]);
+    }
+  }
   const gvx_f4 th = ldtab(&T.hyp[umin32(n, GVX_HYP_N)]);
   const gvx_f4 ts = ldtab(&T.sin[umin32(j, GVX_SIN_N)]);
   const ff2 A = {mk2(th.z, ts.x), mk2(th.w, ts.y)};     // (sinh, sin) of the table point
   const ff2 B = {mk2(th.x, ts.z), mk2(th.y, ts.w)};     // (cosh, cos)
   const ff2 Bn = {mk2(th.z, -ts.x), mk2(th.w, -ts.y)};  // (sinh, -sin)
-  const ff2 r = pack(re, rp);
+  // the leading parts are in steps of 2^-39 and |hi| >= |lo| or hi = 0: normalised for the small ones
+  const ff2 r = fast_two_sum2(mk2(re.hi, rp.hi), mk2(re.lo, rp.lo));
   const TabPoly<f2> tp = tab_poly(r, mk2(0.5f, -0.5f));
   const ff2 w = tab_comb(A, B, r, tp), wc = tab_comb_any(B, Bn, r, tp);
   const ff2 w2 = lc_sqr(w);
   *S = lc_add(lane_x(w2), lane_y(w2));
-  const float se = u2f(0x40800000u | ((uint32_t)(de >> 32) & 0x80000000u));  // +-4
-  const float sp = u2f(0x40800000u | ((uint32_t)(dp >> 32) & 0x80000000u));
-  *sd = lc_scale(lc_mul(w, wc), mk2(se, sp));
-  return S->hi >= kFxMinS;
+  *sd = lc_scale(lc_mul(w, wc), mk2(u2f(0x40800000u | (se & 0x80000000u)), u2f(0x40800000u | (sp & 0x80000000u))));  // +-4
+  return good && (S->hi >= kFxMinS || dp == raw);
 }
 
 // |gm| in [2^-60, 2^20], or gm = 0.
@@ -56,12 +77,15 @@ GVX_HD bool ev_grad_in_range(double g) {
   return hg - (963u << 20) < (81u << 20) || (hg | dlo(g)) == 0u;
 }
 
-// The five terms of a pair, times 2^32; false where the caller has to take the elementwise formulas (S
-// below kFxMinS from angles that are not exact, m^2 nonzero and below 2^-80, gm out of range).
-GVX_HD bool ev_pair_grad(const EvPart &a, const EvPart &b, double g, const LcTab &T, EvGrad *o) {
+// The five terms of a pair, times 2^32 (exact, near: lc_pair_angles_fx); false where the caller has to
+// take the elementwise formulas (angles that the staged ones do not give, m^2 nonzero and below 2^-80,
+// gm out of range).
+template <class Near>
+GVX_HD bool ev_pair_grad(const EvPart &a, const EvPart &b, bool exact, const Near &near, double g, const LcTab &T,
+                         EvGrad *o) {
   ff S;
   ff2 sd;
-  const bool ok = lc_pair_angles_fx(a.eta, a.phi, b.eta, b.phi, T, &S, &sd) || ev_near_exact(a, b);
+  const bool ok = lc_pair_angles_fx(a.eta, a.phi, b.eta, b.phi, exact, near, T, &S, &sd);
   const ff2 s = lc_add(ff2{mk2(a.dy.x, a.dy.y), mk2(a.dy.z, a.dy.w)},
                        ff2{mk2(b.dy.x, b.dy.y), mk2(b.dy.z, b.dy.w)});  // (D_a + D_b, Y_a + Y_b)
   const ff p12 = lc_mul(ff{a.pt_hi, a.pt_lo}, ff{b.pt_hi, b.pt_lo});
@@ -70,7 +94,7 @@ GVX_HD bool ev_pair_grad(const EvPart &a, const EvPart &b, double g, const LcTab
   const uint32_t hg = dhi(g) & 0x7fffffffu;
   if (m2s.hi == 0.0f || (hg | dlo(g)) == 0u) {  // m = 0 or gm = 0: no contribution
     *o = EvGrad{{bc2(0.0f), bc2(0.0f)}, {bc2(0.0f), bc2(0.0f)}, {0.0f, 0.0f}};
-    return ok;
+    return ok && (S.hi == 0.0f || (hg | dlo(g)) == 0u);  // m^2 below the floats is not 0
   }
   const ff m = lc_sqrt_refined(m2s);
   const ff gf = cvt1(cvt_parts(hg, dlo(g), kRebaseOne - kGradShift));
@@ -87,6 +111,10 @@ GVX_HD bool ev_pair_grad(const EvPart &a, const EvPart &b, double g, const LcTab
   o->zu = lc_mul(cb, pack(E2, ta));
   o->vp = lane_y(v);
   return ok && m2s.hi >= 8.27180613e-25f && ev_grad_in_range(g);  // 2^-80
+}
+// The same from the staged particles alone.
+GVX_HD bool ev_pair_grad(const EvPart &a, const EvPart &b, double g, const LcTab &T, EvGrad *o) {
+  return ev_pair_grad(a, b, ev_exact(a.eta, a.phi) && ev_exact(b.eta, b.phi), [](double *) { return false; }, g, T, o);
 }
 
 // ---- a particle's own part --------------------------------------------------------------------

@@ -182,7 +182,11 @@ __device__ __forceinline__ bool stage_particle(const Staged &S, int c, const V4<
     const ffm::ff mmf = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(m), rb));
     const int64_t ae = ffm::angle_fx(eta), ap = ffm::angle_fx(phi);
     uint32_t n, j;
-    const ffm::ff re = ffm::own_reduce(eta, ae, &n), rp = ffm::own_reduce(phi, ap, &j);
+    ffm::ff re = ffm::fx_half_reduce(2 * ae, &n), rp = ffm::fx_half_reduce(2 * ap, &j);
+    if (ffm::fx_small(ae, ap)) {  // seldom
+      re = ffm::own_reduce(eta, ae, &n);
+      rp = ffm::own_reduce(phi, ap, &j);
+    }
     ffm::ff sh, sn, cs;
     const ffm::LcLeg<ffm::ff> L = ffm::lc_leg_at(ptf, mmf, re, &n, T.hyp, &sh);
     S.dy[c] = make_float4(L.D.hi, L.Y.hi, L.D.lo, L.Y.lo);

@@ -165,6 +165,15 @@ __device__ __forceinline__ void big_event(const BArgs &A, const ffm::LcTab &T, i
   }
 }
 
+// Whether a particle's angles are exact travels to the pairs as the last bit of D.lo, 2^-47 of a D that
+// is good to 2^-45.
+__device__ __forceinline__ float mark_inexact(float lo, bool inexact) {
+  return __uint_as_float((__float_as_uint(lo) & ~1u) | (uint32_t)inexact);
+}
+__device__ __forceinline__ bool both_exact(const ffm::EvPart &a, const ffm::EvPart &b) {
+  return ((__float_as_uint(a.dy.z) | __float_as_uint(b.dy.z)) & 1u) == 0u;
+}
+
 // (a) The particles of places c and c + 32 (the second only with `two`) at their events' scale words,
 // as the lanes of paired FP32 instructions.  False where one lies outside the float-float domain.
 __device__ __forceinline__ bool stage_particles(WarpBuf &W, int c, bool two, const V4<double> *x,
@@ -193,7 +202,7 @@ __device__ __forceinline__ bool stage_particles(WarpBuf &W, int c, bool two, con
     const int k = c + 32 * r;
     const ffm::ff D = r ? ffm::lane_y(L.D) : ffm::lane_x(L.D), Y = r ? ffm::lane_y(L.Y) : ffm::lane_x(L.Y);
     const ffm::ff ms = ffm::with_sign(mm[r], ffm::dhi(x[r].w));
-    W.dy[k] = make_float4(D.hi, Y.hi, D.lo, Y.lo);
+    W.dy[k] = make_float4(D.hi, Y.hi, mark_inexact(D.lo, !ffm::ev_exact(ae[r], ap[r])), Y.lo);
     W.ang[k] = make_longlong2(ae[r], ap[r]);
     W.pt[k] = make_float2(ok[r] ? pt[r].hi : -1.0f, pt[r].lo);
     W.mm[k] = make_float2(ms.hi, ms.lo);
@@ -326,7 +335,14 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
         if (GVX_IN_BOUNDS(i, np, A.status) && GVX_IN_BOUNDS(j, np, A.status)) {
           const ffm::EvPart a = staged(W, i), b = staged(W, j);
           ffm::EvGrad o;
-          slow = !ffm::ev_pair_grad(a, b, g, T, &o) || (extreme && (a.pt_hi < 0.0f || b.pt_hi < 0.0f));
+          const auto near = [&](double *d) {
+            const V4<double> u = ld4c<LP>(A.p, pb + i), v = ld4c<LP>(A.p, pb + j);
+            d[0] = u.y - v.y;
+            d[1] = u.z - v.z;
+            return true;
+          };
+          slow = !ffm::ev_pair_grad(a, b, both_exact(a, b), near, g, T, &o) ||
+                 (extreme && (a.pt_hi < 0.0f || b.pt_hi < 0.0f));
           if constexpr (!RARE) {
             if (slow) {
               o = ffm::EvGrad{{ffm::bc2(0.0f), ffm::bc2(0.0f)}, {ffm::bc2(0.0f), ffm::bc2(0.0f)}, {0.0f, 0.0f}};
@@ -407,7 +423,7 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
     const bool fast = p.pt_hi >= 0.0f, done = !A.has_gsum || (fast && ewg != 1u);
     if constexpr (!RARE) {
       ffm::EvOwn<ffm::ff> own = ffm::ev_own(p, ffm::ff{m.x, m.y});
-      if (ffm::fx_small(p.eta) || ffm::fx_small(p.phi)) {  // the angles themselves, seldom
+      if (ffm::fx_small(p.eta, p.phi)) {  // the angles themselves, seldom
         const V4<double> v = ld4c<LP>(A.p, pb + c);
         own.re = ffm::own_reduce(v.y, p.eta, &own.n[0]);
         own.rp = ffm::own_reduce(v.z, p.phi, &own.j[0]);
