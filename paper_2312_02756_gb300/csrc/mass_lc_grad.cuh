@@ -103,8 +103,8 @@ GVX_HD bool pair_mass_grad_lc(double pt1, double eta1, double phi1, double m1, d
   // -- the legs (lane x: leg 1, lane y: leg 2) --
   const ff2 pt = cvt2(cvt_parts(hp1, dlo(pt1), rb), cvt_parts(hp2, dlo(pt2), rb));
   const ff2 mm = cvt2(cvt_parts(hm1, dlo(m1), rb), cvt_parts(hm2, dlo(m2), rb));
-  const ff2 x = cvt2(cvt_parts_normal(umax32(he1, 0x3E100000u), dlo(eta1), kRebaseOne),
-                     cvt_parts_normal(umax32(he2, 0x3E100000u), dlo(eta2), kRebaseOne));
+  // |eta| down to 0 (the forward, which needs cosh alone, raises it to 2^-30): d/deta has sinh for a factor
+  const ff2 x = cvt2(cvt_parts(he1, dlo(eta1), kRebaseOne), cvt_parts(he2, dlo(eta2), kRebaseOne));
   ff2 sh, ch;
   const LcLeg<ff2> L = lc_leg(pt, mm, x, T.hyp, &sh, &ch);
 
