@@ -46,6 +46,15 @@ constexpr int kRaw = 256;     // particles per batch of a warp (eight ballots)
 constexpr int kCap = 128;     // selected particles per run, and particles of an event a warp takes
 constexpr int kMaxTile = 32;  // events per warp tile, at most
 constexpr unsigned kAll = 0xffffffffu;
+// A slot of the CTA's histogram has 32 bits.  At most it takes, between two flushes, the pairs of
+// kMaxTurns tiles of each warp in either walk (the grid is large enough for that), of staged events up to
+// kFlushPairs (and one event more), and of one part of a larger event.
+constexpr int kMaxTurns = 256;
+constexpr long long kFlushPairs = 1ll << 30;
+static_assert(kFlushPairs % kNT == 0 &&
+                  2ll * kWarps * kMaxTurns * kMaxTile * (kCap * (kCap - 1) / 2) + 2 * kFlushPairs +
+                          kNT * (kNT - 1) / 2 < (1ll << 32),
+              "no slot can wrap around");
 
 struct SArgs {
   Lv p;
@@ -93,10 +102,12 @@ __device__ __forceinline__ bool bad_event(const SArgs &A, int64_t e, int64_t lo,
          (e == A.n_events - 1 && hi != A.n_particles);
 }
 
-// A slot of the CTA's histogram added to the caller's counts.
-__device__ __forceinline__ void flush_slot(const SArgs &A, unsigned *s_hist, int s) {
-  if (s_hist[s]) atomicAdd(A.counts + s, (unsigned long long)s_hist[s]);
-  s_hist[s] = 0u;
+// The CTA's histogram moved to the caller's counts, by the whole block with no warp counting meanwhile.
+__device__ __forceinline__ void flush_slots(const SArgs &A, unsigned *s_hist) {
+  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) {
+    if (s_hist[s]) atomicAdd(A.counts + s, (unsigned long long)s_hist[s]);
+    s_hist[s] = 0u;
+  }
 }
 
 // Histogram slot of a mass: 0 below lo, n_bins + 1 at or above hi (and NaN), else 1 + the bin
@@ -196,19 +207,25 @@ __device__ __noinline__ void big_event_select(const SArgs &A, const ffm::LcTab &
   double bd = INFINITY, bm = NAN;
   long long bk = -1;
   const long long npairs = (long long)n * (n - 1) / 2;
-  for (long long k = threadIdx.x; k < npairs; k += kNT) {
-    int64_t i, j;
-    decode_pair_wide(k, n, i, j);
-    const V4<double> x = ld4c<LP>(A.p, pb + i), y = ld4c<LP>(A.p, pb + j);
-    if (!(passes(x.x, x.y, A) && passes(y.x, y.y, A))) continue;
-    const double m = pair_mass_raw(x, y, T);
-    atomicAdd(&s_hist[slot_of(m, A)], 1u);
-    const double d = fabs(m - A.target);
-    if (better(d, k, bd, bk)) {
-      bd = d;
-      bk = k;
-      bm = m;
+  for (long long k0 = 0; k0 < npairs; k0 += kFlushPairs) {
+    const long long k1 = npairs - k0 < kFlushPairs ? npairs : k0 + kFlushPairs;
+    for (long long k = k0 + threadIdx.x; k < k1; k += kNT) {
+      int64_t i, j;
+      decode_pair_wide(k, n, i, j);
+      const V4<double> x = ld4c<LP>(A.p, pb + i), y = ld4c<LP>(A.p, pb + j);
+      if (!(passes(x.x, x.y, A) && passes(y.x, y.y, A))) continue;
+      const double m = pair_mass_raw(x, y, T);
+      atomicAdd(&s_hist[slot_of(m, A)], 1u);
+      const double d = fabs(m - A.target);
+      if (better(d, k, bd, bk)) {
+        bd = d;
+        bk = k;
+        bm = m;
+      }
     }
+    __syncthreads();  // all of these counted before any of the next
+    flush_slots(A, s_hist);
+    __syncthreads();
   }
   *bd_out = bd;
   *bk_out = bk;
@@ -515,6 +532,7 @@ __device__ __noinline__ void finish_tiles(const SArgs &A, unsigned char *s_dyn, 
   if (!__syncthreads_or(large)) return;
   ffm::EvPart *part = reinterpret_cast<ffm::EvPart *>(s_dyn);
   static_assert(sizeof(WarpBuf) * kWarps >= kNT * sizeof(ffm::EvPart), "an event staged by the block");
+  int64_t counted = 0;
   for (int64_t t0 = (int64_t)blockIdx.x * kWarps; t0 < n_tiles; t0 += (int64_t)gridDim.x * kWarps) {
     const int64_t t = t0 + warp;
     const int ne = t < n_tiles ? events_of(A, t) : 0;
@@ -551,9 +569,11 @@ __device__ __noinline__ void finish_tiles(const SArgs &A, unsigned char *s_dyn, 
           if (A.best_m) A.best_m[ev] = bk >= 0 ? bm : NAN;
         }
         __syncthreads();
-        if (n > kNT) {  // so that no slot of the CTA's counts can pass 2^32
-          for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) flush_slot(A, s_hist, s);
+        counted = n > kNT ? 0 : counted + n * (n - 1) / 2;  // big_event_select has flushed
+        if (counted >= kFlushPairs) {
+          flush_slots(A, s_hist);
           __syncthreads();
+          counted = 0;
         }
       }
     }
@@ -597,7 +617,7 @@ __global__ void __launch_bounds__(kNT, 3) pair_select_kernel(const __grid_consta
   }
   if (__syncthreads_or(large || rare != 0)) finish_tiles<LP>(A, s_dyn, s_hist, n_tiles, rare);
   __syncthreads();
-  for (int s = threadIdx.x; s < A.n_bins + 2; s += kNT) flush_slot(A, s_hist, s);
+  flush_slots(A, s_hist);
 }
 
 template <int LP>
@@ -615,7 +635,9 @@ cudaError_t launch_l(SArgs A, cudaStream_t s) {
   A.tile = (int)(want < kMaxTile ? want : kMaxTile);
   const int64_t n_tiles = (A.n_events + A.tile - 1) / A.tile;
   const int64_t need = (n_tiles + kWarps - 1) / kWarps, cap = warps / kWarps;
-  const int64_t grid = need < cap ? need : cap;
+  // the CTAs that fit at once; more where a warp would have more than kMaxTurns tiles (30 M events)
+  const int64_t few = (n_tiles + kWarps * kMaxTurns - 1) / (kWarps * kMaxTurns);
+  const int64_t grid = need < cap ? need : few > cap ? few : cap;
   A.turns = (int)((n_tiles + 64 * grid * kWarps - 1) / (64 * grid * kWarps));
   k<<<(unsigned)grid, kNT, smem, s>>>(A);
   return cudaGetLastError();
