@@ -134,9 +134,10 @@ __device__ __forceinline__ int slot_of_ff(ffm::ff m, float sf, const SArgs &A) {
   return fabsf(t - rintf(t)) > tol ? (int)floorf(t) + 1 : -1;
 }
 
-// (d, k) before (d', k'): the smaller |m - target|, then the smaller k; k < 0 is "none".
+// (d, k) before (d', k'): the smaller |m - target|, NaN last, then the smaller k; k < 0 is "none".  (NaN
+// last, because a thread's first pair may have none while its later ones do.)
 __device__ __forceinline__ bool better(double d, long long k, double d0, long long k0) {
-  return k >= 0 && (k0 < 0 || d < d0 || (d == d0 && k < k0));
+  return k >= 0 && (k0 < 0 || d < d0 || (d == d0 && k < k0) || (isnan(d0) && (!isnan(d) || k < k0)));
 }
 
 // pt and eta of one particle.
