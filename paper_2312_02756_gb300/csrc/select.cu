@@ -30,12 +30,12 @@
 #include <cuda_runtime.h>
 
 #include <math.h>
-#include <string.h>
 
 #include "common.cuh"
 #include "event_lc.cuh"
 #include "pair_index.cuh"
 #include "pair_raw.cuh"
+#include "select_cuts.cuh"
 
 namespace gvx {
 namespace {
@@ -60,8 +60,7 @@ struct SArgs {
   Lv p;
   const int64_t *off;
   int64_t n_events, n_particles;
-  long long pt_lo;                       // the cuts (passes)
-  unsigned long long pt_span, eta_end;
+  Cuts cuts;
   double lo, hi, inv_w, target;
   float lo_h, lo_l, inv_f, tol0;  // the float histogram slot (slot_of_ff)
   int n_bins, tile, turns;        // tile: events per warp tile; turns: a warp's tiles per bit of its rare mask
@@ -83,18 +82,6 @@ struct __align__(16) WarpBuf {
   int pp[32], cs[32], n[32];     // by event: first pair and place in the run, selected particles
   uint32_t scale[32];            // by event: the largest high word of pt and |m|
 };
-
-// The cuts pt >= pt_min and |eta| <= eta_max on the bits of the doubles (an FP64 comparison holds the
-// FP64 pipe like an addition): ordered as signed integers, a double is at least pt_min (and no NaN)
-// when its integer lies in [pt_lo, +inf's]; |eta|'s bits are below eta_end.
-__device__ __forceinline__ long long ordered(double x) {
-  const long long b = __double_as_longlong(x);
-  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-}
-__device__ __forceinline__ bool passes(double pt, double eta, const SArgs &A) {
-  return (unsigned long long)(ordered(pt) - A.pt_lo) <= A.pt_span &&
-         ((unsigned long long)__double_as_longlong(eta) & 0x7fffffffffffffffull) < A.eta_end;
-}
 
 // Offsets lo, hi of event e that cannot be right.
 __device__ __forceinline__ bool bad_event(const SArgs &A, int64_t e, int64_t lo, int64_t hi) {
@@ -214,7 +201,7 @@ __device__ __noinline__ void big_event_select(const SArgs &A, const ffm::LcTab &
       int64_t i, j;
       decode_pair_wide(k, n, i, j);
       const V4<double> x = ld4c<LP>(A.p, pb + i), y = ld4c<LP>(A.p, pb + j);
-      if (!(passes(x.x, x.y, A) && passes(y.x, y.y, A))) continue;
+      if (!(passes(x.x, x.y, A.cuts) && passes(y.x, y.y, A.cuts))) continue;
       const double m = pair_mass_raw(x, y, T);
       atomicAdd(&s_hist[slot_of(m, A)], 1u);
       const double d = fabs(m - A.target);
@@ -245,7 +232,7 @@ __device__ __noinline__ void staged_event_select(const SArgs &A, const ffm::LcTa
   V4<double> x = {0.0, 0.0, 0.0, 0.0};
   const bool in = k < n;
   if (in) x = ld4<double, LP>(A.p, pb + k);
-  const bool pass = in && passes(x.x, x.y, A);
+  const bool pass = in && passes(x.x, x.y, A.cuts);
   if (k == 0) s_scale = 0u;
   int64_t nsel;
   const int c = (int)block_excl_scan<kNT>(pass ? 1 : 0, s_warp, &nsel);  // ends synchronised
@@ -370,7 +357,7 @@ __device__ __forceinline__ int warp_tile(const SArgs &A, const ffm::LcTab &T, Wa
         }
 #pragma unroll
         for (int u = 0; u < 4; u++) {
-          const unsigned b = __ballot_sync(kAll, passes(pt[u], eta[u], A));
+          const unsigned b = __ballot_sync(kAll, passes(pt[u], eta[u], A.cuts));
           if (lane == r / 32 + u) word = b;
         }
       }
@@ -655,17 +642,7 @@ cudaError_t launch_pair_select(const Lv &p, const int64_t *off, int64_t n_events
   A.off = off;
   A.n_events = n_events;
   A.n_particles = n_particles;
-  // the cuts on ordered integers: -0 passes a threshold of 0, nothing passes a NaN
-  const auto bits = [](double x) {
-    long long b;
-    memcpy(&b, &x, sizeof b);
-    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
-  };
-  const long long inf = bits(INFINITY);
-  A.pt_lo = pt_min == 0.0 ? bits(-0.0) : bits(pt_min);
-  A.pt_span = (unsigned long long)inf - (unsigned long long)A.pt_lo;
-  A.eta_end = eta_max >= 0.0 ? (unsigned long long)bits(fabs(eta_max)) + 1ull : 0ull;
-  if (!(pt_min <= INFINITY)) A.eta_end = 0ull;
+  A.cuts = make_cuts(pt_min, eta_max);
   A.lo = lo;
   A.hi = hi;
   A.inv_w = (double)n_bins / (hi - lo);
