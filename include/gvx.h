@@ -242,7 +242,7 @@ gvx_status gvx_event_pair_masses(const gvx_lv *particles, const int64_t *offsets
  *                    contents are scratch; calls in flight at once need separate workspaces.
  * Deterministic (a fixed summation order per particle).  Offsets or pair offsets that do not
  * match the event sizes or n_pairs are detected on the device: GVX_ERR_OFFSETS is recorded in the
- * device status word and the gradients of the affected events are not written.  All pointers
+ * device status word and the gradients of the events they delimit are not written.  All pointers
  * are device (or GPU-addressable host) memory; nothing is allocated.  Two launches: the staged
  * float-float pass, which notes in the workspace what it left of each tile of events (pairs and
  * event-sum parts outside the float-float domain, events of more than 64 particles), then a pass

@@ -29,8 +29,8 @@
 // once more and adding the FP64 formulas to the gradients written; and events with more than kCapW
 // particles, by a CTA straight from global memory with the elementwise adjoint.  The pair offsets
 // are those the forward call wrote; each tile checks them (and the offsets) against the event sizes
-// and the pair count before it reads any pair gradient, and records GVX_ERR_OFFSETS for a tile that
-// does not match (its particles' gradients are then not written).
+// and the pair count before it reads any pair gradient, and records GVX_ERR_OFFSETS where they do not
+// match; of such a tile the second launch does the events whose own offsets are right, each by a CTA.
 //
 // Bound by issue (the first launch; 58% of the slots, held back by dependent chains at 20 warps per SM).
 // 300,007 events, 9.6 M pairs: 382 us both launches, against 550 us for block-wide sub-batches whose
@@ -514,24 +514,24 @@ __device__ __forceinline__ void walk_tile(const BArgs &A, const ffm::LcTab &T, W
   }
 }
 
-constexpr unsigned long long kLarge = 1ull << 32;
+constexpr unsigned long long kLarge = 1ull << 32, kBad = 2ull << 32;
 
-// A tile's offsets into shared memory; false for a tile whose offsets cannot be right.
+// Whether the offsets of event e (particles a .. b - 1, pairs pa .. pb - 1) cannot be right.
+__device__ __forceinline__ bool bad_event(const BArgs &A, int64_t e, int64_t a, int64_t b, int64_t pa, int64_t pb) {
+  const int64_t n = b - a;
+  return a < 0 || n < 0 || b > A.n_particles || n > (1ll << 31) || pa < 0 || pb > A.n_pairs ||
+         pb - pa != n * (n - 1) / 2 || (e == 0 && (a != 0 || pa != 0));
+}
+
+// A tile's offsets into shared memory; false for a tile with an event whose offsets cannot be right.
 __device__ __forceinline__ bool load_tile(const BArgs &A, int64_t e0, int ne, int64_t *s_off, int64_t *s_po) {
   for (int k = threadIdx.x; k <= ne; k += kNT) {
     s_off[k] = A.off[e0 + k];
     s_po[k] = A.pair_off[e0 + k];
   }
   __syncthreads();
-  bool bad = false;
-  if (threadIdx.x < ne) {
-    const int64_t a = s_off[threadIdx.x], b = s_off[threadIdx.x + 1], n = b - a;
-    const int64_t pa = s_po[threadIdx.x], pb = s_po[threadIdx.x + 1];
-    bad = a < 0 || n < 0 || b > A.n_particles || n > (1ll << 31) || pa < 0 || pb > A.n_pairs ||
-          pb - pa != n * (n - 1) / 2;
-    if (e0 + threadIdx.x == 0 && (a != 0 || pa != 0)) bad = true;
-  }
-  return !__syncthreads_or(bad);
+  const int t = threadIdx.x;
+  return !__syncthreads_or(t < ne && bad_event(A, e0 + t, s_off[t], s_off[t + 1], s_po[t], s_po[t + 1]));
 }
 
 template <int LP, int LS, int LG>
@@ -553,8 +553,9 @@ __global__ void __launch_bounds__(kNT, kCtas) event_pairs_bwd_kernel(const __gri
       walk_tile<LP, LS, LG, false>(A, T, bufs[threadIdx.x >> 5], s_tile, e0, ne, s_off, s_po, &large);
       __syncthreads();
       left = s_tile.rare | (large ? kLarge : 0ull);
-    } else if (threadIdx.x == 0) {
-      raise_status(A.status, GVX_ERR_OFFSETS);
+    } else {
+      left = kBad;
+      if (threadIdx.x == 0) raise_status(A.status, GVX_ERR_OFFSETS);
     }
     if (threadIdx.x == 0) A.left[tile] = left;
   }
@@ -587,14 +588,17 @@ __global__ void __launch_bounds__(kNT, 4) event_pairs_bwd_left_kernel(const __gr
       const int ne = (int)(A.n_events - e0 < A.te ? A.n_events - e0 : A.te);
       __syncthreads();  // the previous tile is done with the shared arrays
       if (threadIdx.x == 0) s_tile = {0, (unsigned)left};
-      if (!load_tile(A, e0, ne, s_off, s_po)) continue;
+      load_tile(A, e0, ne, s_off, s_po);
       bool large;
       if ((unsigned)left != 0u)
         walk_tile<LP, LS, LG, true>(A, T, bufs[threadIdx.x >> 5], s_tile, e0, ne, s_off, s_po, &large);
-      if (left & kLarge)
-        for (int e = 0; e < ne; e++)
-          if (s_off[e + 1] - s_off[e] > kCapW)
-            big_event<LP, LS, LG>(A, T, e0 + e, s_off[e], s_off[e + 1] - s_off[e], s_po[e]);
+      if (left & (kLarge | kBad))
+        for (int e = 0; e < ne; e++) {
+          const int64_t pbeg = s_off[e], n = s_off[e + 1] - pbeg;
+          // of a tile with malformed offsets, every event whose own are right
+          if ((left & kBad) ? !bad_event(A, e0 + e, pbeg, pbeg + n, s_po[e], s_po[e + 1]) : n > kCapW)
+            big_event<LP, LS, LG>(A, T, e0 + e, pbeg, n, s_po[e]);
+        }
     }
     __syncthreads();
   }
