@@ -561,9 +561,13 @@ __global__ void __launch_bounds__(kNT, kCtas) event_pairs_bwd_kernel(const __gri
   }
 }
 
-// What the first launch left (nothing, most of the time): every block scans its part of the tiles'
-// words and takes the tiles that have one.  A launch of its own, because a call anywhere in the first
-// kernel costs its batches spills (413 us against 392 us at 300,007 events).
+// What the first launch left (nothing, most of the time): every block scans its share of the tiles'
+// words and takes what they note.  A launch of its own, because a call anywhere in the first kernel
+// costs its batches spills (413 us against 392 us at 300,007 events).  A tile counts kParts times, for
+// its flagged batches and for every kParts-th of its large events, so that a few tiles of large events
+// still reach all SMs (2,000 events of 150 particles: 2,284 us, by whole tiles 6,809 us).
+constexpr int kParts = 8;
+
 template <int LP, int LS, int LG>
 __global__ void __launch_bounds__(kNT, 4) event_pairs_bwd_left_kernel(const __grid_constant__ BArgs A) {
   extern __shared__ __align__(16) unsigned char s_dyn[];
@@ -573,18 +577,19 @@ __global__ void __launch_bounds__(kNT, 4) event_pairs_bwd_left_kernel(const __gr
   __shared__ unsigned long long s_left[kNT];
   const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
   const int64_t n_tiles = (A.n_events + A.te - 1) / A.te;
-  // the block's tiles: every gridDim.x-th, a thread looking at one (so that neighbouring tiles, often
+  // the block's share: every gridDim.x-th, a thread looking at one (so that neighbouring tiles, often
   // alike, go to different blocks)
-  for (int64_t t0 = blockIdx.x; t0 < n_tiles; t0 += (int64_t)gridDim.x * kNT) {
+  for (int64_t t0 = blockIdx.x; t0 < kParts * n_tiles; t0 += (int64_t)gridDim.x * kNT) {
     const int64_t t = t0 + (int64_t)gridDim.x * threadIdx.x;
-    const unsigned long long mine = t < n_tiles ? A.left[t] : 0ull;
+    unsigned long long mine = t < kParts * n_tiles ? A.left[t % n_tiles] : 0ull;
+    if (t >= n_tiles) mine &= kLarge | kBad;  // the batches are part 0's
     if (!__syncthreads_or(mine != 0ull)) continue;
     s_left[threadIdx.x] = mine;
     __syncthreads();
     for (int k = 0; k < kNT; k++) {
       const unsigned long long left = s_left[k];
       if (left == 0ull) continue;
-      const int64_t e0 = (t0 + (int64_t)gridDim.x * k) * A.te;
+      const int64_t item = t0 + (int64_t)gridDim.x * k, e0 = item % n_tiles * A.te;
       const int ne = (int)(A.n_events - e0 < A.te ? A.n_events - e0 : A.te);
       __syncthreads();  // the previous tile is done with the shared arrays
       if (threadIdx.x == 0) s_tile = {0, (unsigned)left};
@@ -593,7 +598,7 @@ __global__ void __launch_bounds__(kNT, 4) event_pairs_bwd_left_kernel(const __gr
       if ((unsigned)left != 0u)
         walk_tile<LP, LS, LG, true>(A, T, bufs[threadIdx.x >> 5], s_tile, e0, ne, s_off, s_po, &large);
       if (left & (kLarge | kBad))
-        for (int e = 0; e < ne; e++) {
+        for (int e = (int)(item / n_tiles); e < ne; e += kParts) {
           const int64_t pbeg = s_off[e], n = s_off[e + 1] - pbeg;
           // of a tile with malformed offsets, every event whose own are right
           if ((left & kBad) ? !bad_event(A, e0 + e, pbeg, pbeg + n, s_po[e], s_po[e + 1]) : n > kCapW)
@@ -629,7 +634,7 @@ cudaError_t launch_l(BArgs A, cudaStream_t s) {
   k<<<balanced_grid_of<k>(kNT, kDynSmem, n_tiles, 1), kNT, kDynSmem, s>>>(A);  // one tile per CTA and pass
   err = cudaGetLastError();
   if (err != cudaSuccess) return err;
-  left<<<balanced_grid_of<left>(kNT, kDynSmem, n_tiles, 1, 1), kNT, kDynSmem, s>>>(A);
+  left<<<balanced_grid_of<left>(kNT, kDynSmem, kParts * n_tiles, 1, 1), kNT, kDynSmem, s>>>(A);
   return cudaGetLastError();
 }
 
