@@ -636,7 +636,7 @@ def run_gvx(args):
 # while these match; gvx_internal.h, which only declares the host-side launch functions, is left
 # out).
 _MASS_SRC = ("mass.cu", "mass_lc.cuh", "mass_lc_grad.cuh", "ff2.cuh", "ff_tables.cuh", "ff.cuh",
-             "pair_math.cuh", "common.cuh", "../gen_tables.py")
+             "pair_math.cuh", "pair_raw.cuh", "common.cuh", "../gen_tables.py")
 KERNEL_SOURCES = {
     "mass_f64_soa": _MASS_SRC,
     "mass_f64_aos": _MASS_SRC,
