@@ -19,15 +19,16 @@ namespace ffm {
 constexpr float kFxMinS = 2.384185791015625e-07f;  // 2^-22
 
 // x, |x| < 8, in units of 2^-59, rounded to nearest (ties away from zero), a nonzero x to at least one
-// unit: 0 stands for 0 alone, and the sign is kept.
+// unit: 0 stands for 0 alone (or |x| < 2^-1042), and the sign is kept.
 GVX_HD int64_t angle_fx(double x) {
   const uint32_t wh = dhi(x), wl = dlo(x);
   // the significand with one guard bit, at the place it has for x in [4, 8)
   const uint64_t M = (((uint64_t)((wh & 0xfffffu) | 0x100000u) << 32) | wl) << 10;
-  const uint32_t sh = 1025u - ((wh >> 20) & 0x7ffu);
+  // |x| raised to 2^-60; 0 wraps around and stays
+  const uint32_t h = umax32((wh & 0x7fffffffu) - 1u, (963u << 20) - 1u) + 1u;
+  const uint32_t sh = 1025u - (h >> 20);
   const uint64_t v = sh < 64u ? M >> sh : 0;
-  int64_t r = (int64_t)((v + 1) >> 1);
-  if (r == 0 && ((wh << 1) | wl) != 0u) r = 1;
+  const int64_t r = (int64_t)((v + 1) >> 1);
   return (wh >> 31) ? -r : r;
 }
 
@@ -125,11 +126,13 @@ GVX_HD bool ev_pair_m2(const EvPart &a, const EvPart &b, const LcTab &T, ff *m2s
 }
 
 // Whether a staged angle is the FP64 one exactly: its last bit is at least 2^-59 from 2^-7 on.
-GVX_HD bool fx_exact(int64_t a) { return (a < 0 ? -a : a) >= (1ll << 52) || a == 0; }
+GVX_HD bool fx_exact(int64_t a) { return (a < 0 ? -a : a) > (1ll << 52) || a == 0; }
 
 
-// Whether both angles of a staged particle are exact.
+// Whether both angles of a staged particle are exact, from them or from the high words of |eta| and |phi|
+// (0 wraps around).
 GVX_HD bool ev_exact(int64_t eta, int64_t phi) { return fx_exact(eta) && fx_exact(phi); }
+GVX_HD bool ev_exact(uint32_t he, uint32_t hf) { return umin32(he - 1u, hf - 1u) >= (1016u << 20) - 1u; }
 
 }  // namespace ffm
 }  // namespace gvx

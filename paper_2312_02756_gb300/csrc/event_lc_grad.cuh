@@ -44,7 +44,7 @@ GVX_HD bool lc_pair_angles_fx(int64_t eta1, int64_t phi1, int64_t eta2, int64_t 
   ff re = fx_half_reduce(de, &n), rp = fx_half_reduce(dp, &j);
   uint32_t se = (uint32_t)(de >> 32), sp = (uint32_t)(dp >> 32);
   bool good = true;
-  if (!exact && fx_small(de, dp)) {
+  if (__builtin_expect((int)fx_small(de, dp) & (int)!exact, 0)) {
     double d[2] = {0.0, 0.0};
     good = near(d);
     if (fx_small(de)) {

@@ -178,15 +178,16 @@ __device__ __forceinline__ bool both_exact(const ffm::EvPart &a, const ffm::EvPa
 // as the lanes of paired FP32 instructions.  False where one lies outside the float-float domain.
 __device__ __forceinline__ bool stage_particles(WarpBuf &W, int c, bool two, const V4<double> *x,
                                                 const uint32_t *wmax, const ffm::LcTab &T) {
-  bool ok[2];
+  bool ok[2], exact[2];
   ffm::ff pt[2], mm[2], re[2];
   int64_t ae[2], ap[2];
   uint32_t n[2];
 #pragma unroll
   for (int r = 0; r < 2; r++) {
     const uint32_t hp = ffm::dhi(x[r].x), hm = ffm::dhi(x[r].w) & 0x7fffffffu;
-    ok[r] = hp >= 0x100000u && ffm::lc_in_domain(hp, hm, ffm::dhi(x[r].y) & 0x7fffffffu,
-                                                 ffm::dhi(x[r].z) & 0x7fffffffu, wmax[r]);
+    const uint32_t he = ffm::dhi(x[r].y) & 0x7fffffffu, hf = ffm::dhi(x[r].z) & 0x7fffffffu;
+    ok[r] = hp >= 0x100000u && ffm::lc_in_domain(hp, hm, he, hf, wmax[r]);
+    exact[r] = ffm::ev_exact(he, hf);
     const uint32_t rb = (wmax[r] & 0x7ff00000u) - (127u << 20);
     pt[r] = ffm::cvt1(ffm::cvt_parts(hp, ffm::dlo(x[r].x), rb));
     mm[r] = ffm::cvt1(ffm::cvt_parts(hm, ffm::dlo(x[r].w), rb));
@@ -202,7 +203,7 @@ __device__ __forceinline__ bool stage_particles(WarpBuf &W, int c, bool two, con
     const int k = c + 32 * r;
     const ffm::ff D = r ? ffm::lane_y(L.D) : ffm::lane_x(L.D), Y = r ? ffm::lane_y(L.Y) : ffm::lane_x(L.Y);
     const ffm::ff ms = ffm::with_sign(mm[r], ffm::dhi(x[r].w));
-    W.dy[k] = make_float4(D.hi, Y.hi, mark_inexact(D.lo, !ffm::ev_exact(ae[r], ap[r])), Y.lo);
+    W.dy[k] = make_float4(D.hi, Y.hi, mark_inexact(D.lo, !exact[r]), Y.lo);
     W.ang[k] = make_longlong2(ae[r], ap[r]);
     W.pt[k] = make_float2(ok[r] ? pt[r].hi : -1.0f, pt[r].lo);
     W.mm[k] = make_float2(ms.hi, ms.lo);
@@ -423,7 +424,7 @@ __device__ __forceinline__ bool warp_batch(const BArgs &A, const ffm::LcTab &T, 
     const bool fast = p.pt_hi >= 0.0f, done = !A.has_gsum || (fast && ewg != 1u);
     if constexpr (!RARE) {
       ffm::EvOwn<ffm::ff> own = ffm::ev_own(p, ffm::ff{m.x, m.y});
-      if (ffm::fx_small(p.eta, p.phi)) {  // the angles themselves, seldom
+      if (__builtin_expect(ffm::fx_small(p.eta, p.phi), 0)) {  // the angles themselves, seldom
         const V4<double> v = ld4c<LP>(A.p, pb + c);
         own.re = ffm::own_reduce(v.y, p.eta, &own.n[0]);
         own.rp = ffm::own_reduce(v.z, p.phi, &own.j[0]);

@@ -30,7 +30,8 @@ extern "C" void enh_pairs(const double *a, const double *b, const double *g, int
     for (int k = 0; k < 4; k++) ga[4 * i + k] = gb[4 * i + k] = NAN;
     ok[i] = asked[i] = 0;
     if (!stage(x, wmax, T, &p, &mp) || !stage(y, wmax, T, &q, &mq)) continue;
-    const bool exact = ev_exact(p.eta, p.phi) && ev_exact(q.eta, q.phi);
+    const auto exact_words = [](const double *v) { return ev_exact(dhi(v[1]) & 0x7fffffffu, dhi(v[2]) & 0x7fffffffu); };
+    const bool exact = exact_words(x) && exact_words(y);
     ok[i] = ev_pair_grad(p, q, exact, [&](double *d) {
       d[0] = x[1] - y[1];
       d[1] = x[2] - y[2];
