@@ -138,12 +138,14 @@ gvx_status gvx_boost(const gvx_lv *v, const gvx_lv *beta, int64_t beta_stride, g
  * GVX_PXPYPZM (px, py, pz, m; E = sqrt(|p|^2 + m^2)) or GVX_PTETAPHIE (pt, eta, phi, E).  A spacelike sum gives -sqrt of
  * |E^2 - |P|^2| (GenVector's convention).  PxPyPzE: the definition evaluated exactly in
  * fixed-point integers (every component truncated to 2^-83 of the pair's largest), within 2^-44
- * relative; PxPyPzM: p1 x p2, p1.p2, |p_i|^2 and m_i^2 in fixed point at each leg's own scale and
- * the cancellation-free combination m1^2 + m2^2 + 2 (E1 E2 - p1.p2) in float-float, within 2^-43
- * relative.  Pairs whose |m^2| falls below 2^-31 of the larger leg's squared scale (a power of
- * two within 2x of its largest component), or outside the fixed-point range, take a
- * cancellation-free FP64 form (an FMA-exact cross product and E^2 - |p|^2): within 1e-12
- * relative for legs with E^2 >= |p|^2.  FP32 legs go through the same evaluations and are rounded
+ * relative; PxPyPzM: the cancellation-free combination m1^2 + m2^2 + 2 (E1 E2 - p1.p2) in
+ * float-float, each leg at its own scale, with p2 reduced by its projection on p1 (one FP64 FMA per
+ * component), within 2^-43 relative.  A pair takes a cancellation-free FP64 form (an FMA-exact cross
+ * product and E^2 - |p|^2; within 1e-12 relative for legs with E^2 >= |p|^2) where its |m^2| falls
+ * below 2^-31 of the larger leg's squared scale (a power of two within 2x of its largest component),
+ * where a scale exponent lies beyond +-900 (FP32 +-100; PxPyPzM +-450 and +-50), where the scales of
+ * two PxPyPzM legs are more than 60 binades apart, or for a denormal FP32 component of a PxPyPzE
+ * pair below scale exponent -43.  FP32 legs go through the same evaluations and are rounded
  * once.  PtEtaPhiE: in FP64 the PtEtaPhiM identity with q_i = E_i^2 - (pt_i cosh eta_i)^2 in
  * float-float; outside its domain (negative E, m^2 below 2^-80 of the scale, spacelike sums) and
  * in FP32, both legs converted to PxPyPzE as gvx_to_pxpypze does and the exact fixed-point mass of
