@@ -88,10 +88,11 @@ __global__ void __launch_bounds__(256) mass_f32_x4_kernel(Lv a, Lv b, float *__r
 }
 
 // FP64 forward: grid-stride, one pair per thread and step; 64 registers, eight CTAs of 128
-// threads per SM, a grid of 32 times the resident CTAs (small CTAs and many waves even out the
-// SMs' progress: 2-3% faster than four CTAs of 256 and 8 waves on GB300).  For a leg in SoA layout (four separate arrays), lanes 0..7 of each warp
-// first ask L2 to prefetch the warp's next 32 elements of each array (one 128-byte line per
-// lane), so that the next step's eight loads find them in L2 rather than in HBM.
+// threads per SM, a grid of up to 32 times the resident CTAs (kMassWaves, kMassSteps; small CTAs and
+// many waves even out the SMs' progress: 2-3% faster than four CTAs of 256 and 8 waves on GB300).  For a
+// leg in SoA layout (four separate arrays), lanes 0..15 of each warp first ask L2 to prefetch the
+// warp's next 32 elements of each array (two 128-byte lines an array, one per lane), so that the next
+// step's eight loads find them in L2 rather than in HBM.
 template <int LA, int LB>
 __global__ void __launch_bounds__(128, 8) mass_f64_kernel(Lv a, Lv b, double *__restrict__ m, int64_t n) {
   const ffm::LcTab T{ffm::kHypTab, ffm::kSinTab};
