@@ -8,7 +8,9 @@
 // route issues about as many instructions and leaves that pipe idle.  A difference carries about
 // 2^-59 of rounding from its two angles, so S = sinh^2(d_eta/2) + sin^2(d_phi/2) keeps 2^-47
 // relative where it is at least 2^-22 (kFxMinS); nearer pairs go to the elementwise arithmetic,
-// which subtracts the angles in FP64.
+// which subtracts the angles in FP64.  What a small angle or difference enters by itself (a
+// particle's components and their gradients, d/deta and d/dphi of a pair) is formed from the doubles
+// below 2^-12 (own_reduce, event_lc_grad.cuh).
 #pragma once
 
 #include "mass_lc.cuh"

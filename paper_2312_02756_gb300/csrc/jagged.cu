@@ -24,9 +24,9 @@
 //      staged the same way up to kCP particles, straight from global memory beyond.
 // Tile descriptors are 64-bit words: 2 flag bits (aggregate / inclusive prefix) + 62-bit value.
 //
-// Bound by issue and the shared-memory/L1 data pipe together (440 warp instructions and 104 data
+// Bound by issue and the shared-memory/L1 data pipe together (445 warp instructions and 104 data
 // wavefronts per 32 pairs, of which the two table gathers take about 40).  2^20 events, 33.5 M
-// pairs: 0.558 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
+// pairs: 0.56 ms a call, against 0.744 ms for block-wide sub-batches with FP64 angle differences
 // and a search per pair (620 instructions per 32 pairs, FP64 pipe 35% busy).  Six CTAs of 128
 // threads per SM (80 registers): eight (64 registers, 0.623 ms) leave the tables too little L1.
 // Tiles of 64 events on 128 threads: 0.615 ms; 256 on 256: 0.587 ms.

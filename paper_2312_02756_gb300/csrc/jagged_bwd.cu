@@ -15,16 +15,20 @@
 //       (event_lc.cuh);
 //   (b) in chunks of kPC pairs, one lane per pair: the five numbers of event_lc_grad.cuh, which
 //       enter both legs' gradients with a sign only, into the pair's slot.  The pairs are taken by
-//       their distance: row t of an event of n particles holds the pairs (i, i + t modulo n);
+//       their distance: row t of an event of n particles holds the pairs (i, i + t modulo n).  A
+//       difference below 2^-12 between angles that are not exact in fixed point (one pair in 10^6) is
+//       taken in FP64 from the particles at once: left to the second launch, such a pair costs that
+//       launch 35 us of latency;
 //   (c) after each chunk, one lane per particle: its signed sums over its pairs of the chunk, two per
 //       row, in a fixed order, so that the result does not depend on scheduling and no atomic
 //       operation touches it.  With the pairs in that order the lanes of an event read
 //       neighbouring slots;
 //   (d) per particle: its gradient from the sums, and J^T gs, both in float-float, converted by
-//       integer operations and added in FP64.
+//       integer operations and added in FP64; sinh(eta) and sin(phi) of an angle below 2^-12 from the
+//       particle itself.
 // What that leaves is noted in a word per tile in the workspace and done by a second launch: pairs
 // outside the float-float domain (either particle outside the forward's domain at the event's scale
-// or with pt = 0, near-equal directions whose difference is not exact, a scaled m^2 below 2^-80, |gm|
+// or with pt = 0, directions near each other across phi = +-pi, a scaled m^2 below 2^-80, |gm|
 // outside [2^-60, 2^20]) and event-sum parts with gs out of range, by walking the batches that met one
 // once more and adding the FP64 formulas to the gradients written; and events with more than kCapW
 // particles, by a CTA straight from global memory with the elementwise adjoint.  The pair offsets
@@ -32,8 +36,9 @@
 // and the pair count before it reads any pair gradient, and records GVX_ERR_OFFSETS where they do not
 // match; of such a tile the second launch does the events whose own offsets are right, each by a CTA.
 //
-// Bound by issue (the first launch; 58% of the slots, held back by dependent chains at 20 warps per SM).
-// 300,007 events, 9.6 M pairs: 382 us both launches, against 550 us for block-wide sub-batches whose
+// Bound by issue (the first launch; 66% of the slots, held back by dependent chains at 20 warps per SM).
+// 300,007 events, 9.6 M pairs: 395 us both launches (382 us before the small angles and differences of
+// (b) and (d), which the figures below leave out), against 550 us for block-wide sub-batches whose
 // particles walked their partners (seven sums of products per direction, 1,150 warp instructions per
 // 32 pairs) and a second launch over every tile with a pair near 2 pi.  By step: pairs in packed
 // order, whose lanes read slots far apart, 465 us; by distance 413; without a call in the first
